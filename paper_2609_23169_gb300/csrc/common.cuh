@@ -62,15 +62,15 @@ UT_DEV bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Bounded wait: returns false (and records UT_ERR_TIMEOUT, raises the CTA's
-// abort flag) if the phase with this parity has not completed within
+// Slow path of a bounded wait: returns false (and records UT_ERR_TIMEOUT, raises
+// the CTA's abort flag) if the phase with this parity has not completed within
 // timeout_ns, or if another role of the CTA has already aborted.  A limit of 0
 // gives up at the first wait that is not already satisfied (diagnostics).
 // The spin loop lives inside one asm block: a loop written in C++ around the
 // wait, placed between tcgen05.mma groups, keeps the tensor pipe from
 // streaming consecutive MMAs (measured: ~2x fewer MMAs per cycle).
-UT_DEV bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
-                      uint64_t timeout_ns) {
+UT_DEV bool mbar_wait_slow(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
+                           uint64_t timeout_ns) {
   uint32_t r;  // 1 = phase complete, 0 = timed out, 2 = CTA already aborted
   asm volatile(
       "{\n\t"
@@ -112,6 +112,14 @@ UT_DEV bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, 
   return false;
 }
 
+// Bounded wait of one thread.  A wait whose phase has already completed, the
+// common case in a pipeline that keeps up, is one try_wait and a branch.
+UT_DEV bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
+                      uint64_t timeout_ns) {
+  if (mbar_try_wait(bar, parity)) return true;
+  return mbar_wait_slow(bar, parity, abort_flag, status, timeout_ns);
+}
+
 // Unbounded-count but time-bounded drain wait (no abort check): used on the way
 // out of a kernel for the CTA's own copies and MMAs.
 UT_DEV bool mbar_drain(uint64_t* bar, uint32_t parity, uint64_t timeout_ns) {
@@ -143,7 +151,11 @@ UT_DEV bool mbar_drain(uint64_t* bar, uint32_t parity, uint64_t timeout_ns) {
 // tcgen05 instructions convergent).
 UT_DEV bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                       uint64_t timeout_ns) {
-  bool r = mbar_wait(bar, parity, abort_flag, status, timeout_ns);
+  // one try_wait and one vote when the phase has completed (43 cycles; through
+  // the slow path's outcome codes a satisfied wait cost 90)
+  bool r = mbar_try_wait(bar, parity);
+  if (__all_sync(0xffffffffu, r)) return true;
+  r = r || mbar_wait_slow(bar, parity, abort_flag, status, timeout_ns);
   return __all_sync(0xffffffffu, r);
 }
 
