@@ -320,7 +320,10 @@ ut_status ut_bsattn_fwd(const ut_attn_shape* shape, const void* q, const void* k
  *   ws          ut_bsattn_bwd_workspace_size(shape) bytes: D and LSE*log2(e)
  *               per head and padded row, and for bf16 an fp32 dQ accumulator
  *               [H, ceil(N/128)*128, d] (about 4*H*N*d bytes) followed by
- *               the counter that hands key blocks to the kernel's CTAs.
+ *               the counter that hands key blocks to the kernel's CTAs and the
+ *               order it hands them out in (4 bytes per 128 rows and head; a
+ *               workspace without these last bytes is accepted, the blocks
+ *               are then handed out in index order).
  * bf16 runs one fused tensor-core kernel per key block (S and dP computed
  * once per retained pair); dQ is summed over key blocks with fp32 atomic
  * additions, so its last bits may differ between runs (dK, dV do not). */

@@ -337,7 +337,7 @@ size_t ut_bsattn_bwd_workspace_size(const ut_attn_shape* shape) {
   int nq = 0, nk = 0;
   if (check_shape(shape, &nq, &nk) != UT_OK) return 0;
   const AttnProblem p = attn_problem(shape, nq, nk, 1.f);
-  const size_t a = attn_bwd_simt_ws(p), b = attn_bwd_tc_ws(p);
+  const size_t a = attn_bwd_simt_ws(p), b = attn_bwd_tc_ws_ordered(p);
   return (a > b ? a : b) + 256;
 }
 
@@ -366,7 +366,7 @@ ut_status ut_bsattn_bwd(const ut_attn_shape* shape, const void* q, const void* k
       !aligned16(dk) || !aligned16(dv))
     return UT_ERR_INVALID_ARG;
   return from_cuda(launch_attn_bwd_tc(p, q, k, v, o, lse, dout, row_ptr, col_idx, col_ptr_t, row_idx_t, dq, dk, dv,
-                                      ws, dev_status, wait_timeout_ns(), device_sms(), s));
+                                      ws, ws_bytes, dev_status, wait_timeout_ns(), device_sms(), s));
 }
 
 }  // extern "C"

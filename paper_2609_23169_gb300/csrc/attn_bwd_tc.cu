@@ -35,13 +35,92 @@ constexpr int kTile = 128;
 constexpr uint32_t kChunk = 128 * 128;  // one 128-row x 128-byte swizzled sub-tile
 
 // ------------------------------------------------------------- preprocess
-// One warp per (padded) row r; a half-warp per head (8 bf16 per lane).
+// Order in which the fused kernel's items (128-row key tiles) are handed out:
+// groups of heads one after another, inside a group the longest lists first.
+// Structured lists differ a lot in length (at the 512 canvas the reference
+// image's key blocks list 61 query blocks, most others 11), and an item taken
+// last holds one CTA while the others are done: handed out in index order the
+// busiest of 152 CTAs had 242 steps against a mean of 199 there (1,516 against
+// 1,388 at 1024), longest first 205 (1,407); a training layer at 1024 went from
+// 5,316 to 5,151 us, at 512 with d = 64 from 440 to 419, this kernel also
+// clearing the accumulator in place of a memset.  A group is as many heads as keep
+// Q, dO and the dQ accumulator (8 N d bytes a head) within kOrderGroupBytes, so
+// that the CTAs in flight still share one group's tiles in L2.
+constexpr int64_t kOrderGroupBytes = 64ll << 20;
+constexpr int kOrderBins = 1024;
+
+struct OrderParams {
+  const int32_t* ptr;  // transposed fine lists
+  int32_t* order;      // [H * nt] (nullptr: index order)
+  int32_t* counter;    // item counter, zeroed here
+  int H, nt, nk_fine, k_rows_per_tile, heads_per_group, groups;
+};
+
+// One CTA per group: a counting sort by list length (which of two equally long
+// items comes first does not matter).
+UT_DEV void order_group(const OrderParams& o, int g) {
+  __shared__ int32_t bins[kOrderBins];
+  __shared__ int32_t warp_tot[8], s_max;
+  const int h0 = g * o.heads_per_group, h1 = min(o.H, h0 + o.heads_per_group);
+  const int first = h0 * o.nt, n = (h1 - h0) * o.nt;
+  auto length = [&](int x) {  // listed blocks of item first + x
+    const int h = h0 + x / o.nt, j = x % o.nt;
+    const int64_t r = (int64_t)h * o.nk_fine + j * o.k_rows_per_tile;
+    const int rows = min(o.k_rows_per_tile, o.nk_fine - j * o.k_rows_per_tile);
+    return o.ptr[r + rows] - o.ptr[r];
+  };
+  if (threadIdx.x == 0) s_max = 1;
+  for (int b = threadIdx.x; b < kOrderBins; b += blockDim.x) bins[b] = 0;
+  __syncthreads();
+  int mx = 1;
+  for (int x = threadIdx.x; x < n; x += blockDim.x) mx = max(mx, length(x));
+  atomicMax(&s_max, mx);
+  __syncthreads();
+  const float inv = (float)(kOrderBins - 1) / (float)s_max;
+  auto bin = [&](int x) { return kOrderBins - 1 - min(kOrderBins - 1, (int)((float)length(x) * inv)); };
+  for (int x = threadIdx.x; x < n; x += blockDim.x) atomicAdd(&bins[bin(x)], 1);
+  __syncthreads();
+  // exclusive prefix of the bins, four per thread (256 threads)
+  const int b0 = threadIdx.x * (kOrderBins / 256), lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  int c[kOrderBins / 256], local = 0;
+#pragma unroll
+  for (int e = 0; e < kOrderBins / 256; ++e) {
+    c[e] = bins[b0 + e];
+    local += c[e];
+  }
+  int incl = local;
+  for (int off = 1; off < 32; off <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += v;
+  }
+  if (lane == 31) warp_tot[wp] = incl;
+  __syncthreads();
+  int run = incl - local;
+  for (int i = 0; i < wp; ++i) run += warp_tot[i];
+#pragma unroll
+  for (int e = 0; e < kOrderBins / 256; ++e) {
+    bins[b0 + e] = run;
+    run += c[e];
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < n; x += blockDim.x) o.order[first + atomicAdd(&bins[bin(x)], 1)] = first + x;
+}
+
+// D_r = dO_r . O_r and LSE_r * log2(e) into the padded [H, Np] workspace, and the
+// dQ accumulator's row cleared; one warp per row r of Np.  The first
+// o.groups blocks write the item order instead.
 __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __restrict__ o,
                                                       const __nv_bfloat16* __restrict__ dout,
                                                       const float* __restrict__ lse, int64_t N, int64_t Np, int H,
                                                       int d, int64_t rs, float* __restrict__ lse2,
-                                                      float* __restrict__ dsum) {
-  const int64_t r = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+                                                      float* __restrict__ dsum, float* __restrict__ dq_acc,
+                                                      const OrderParams op) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *op.counter = 0;
+  if ((int)blockIdx.x < op.groups) {
+    order_group(op, blockIdx.x);
+    return;
+  }
+  const int64_t r = (int64_t)(blockIdx.x - op.groups) * 8 + (threadIdx.x >> 5);
   if (r >= Np) return;
   const int lane = threadIdx.x & 31;
   const int lanes_per_head = d / 8;           // 16 (d=128) or 8 (d=64)
@@ -62,6 +141,11 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
         s = fmaf(x.x, y.x, s);
         s = fmaf(x.y, y.y, s);
       }
+    }
+    if (h < H) {
+      uint4* acc = reinterpret_cast<uint4*>(dq_acc + ((int64_t)h * Np + r) * d + (lane % lanes_per_head) * 8);
+      acc[0] = make_uint4(0, 0, 0, 0);
+      acc[1] = make_uint4(0, 0, 0, 0);
     }
     for (int off = lanes_per_head / 2; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if ((lane % lanes_per_head) == 0 && h < H) {
@@ -87,6 +171,7 @@ struct BwdParams {
   float scale, scale_log2;
   uint64_t timeout_ns;
   int32_t* item_counter;  // next item to hand out (zeroed before the launch)
+  const int32_t* order;   // the items in the order they are handed out (nullptr: index order)
 };
 
 // 64 consecutive TMEM columns of this warp's 32 lanes, one wait.
@@ -279,6 +364,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
             if (!(ok = mbar_wait(&sm.item_empty[s], (n & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns))) break;
             w = atomicAdd(prm.item_counter, 1);
             if (w >= prm.n_items) w = -1;
+            else if (prm.order) w = prm.order[w];
             *reinterpret_cast<volatile int32_t*>(&sm.item[s]) = w;
             mbar_arrive(&sm.item_full[s]);
             ++kk;
@@ -664,9 +750,17 @@ __global__ void __launch_bounds__(256) bwd_dq_finalize_kernel(const float* __res
 }
 
 // ----------------------------------------------------------------- launcher
+static size_t bwd_tiles(const AttnProblem& p) { return (size_t)((p.N + kTile - 1) / kTile); }
+
 size_t attn_bwd_tc_ws(const AttnProblem& p) {
-  const size_t Np = (size_t)((p.N + kTile - 1) / kTile) * kTile;
+  const size_t Np = bwd_tiles(p) * kTile;
   return 2 * (size_t)p.H * Np * sizeof(float) + (size_t)p.H * Np * p.d * sizeof(float) + 16;  // + item counter
+}
+
+// With the item order after the counter; a smaller workspace (at least
+// attn_bwd_tc_ws) hands the items out in index order.
+size_t attn_bwd_tc_ws_ordered(const AttnProblem& p) {
+  return attn_bwd_tc_ws(p) + (size_t)p.H * bwd_tiles(p) * sizeof(int32_t);
 }
 
 constexpr size_t kMaxDynSmem = 232448;  // 227 KB opt-in per block on sm_100/sm_103
@@ -699,7 +793,8 @@ static cudaError_t launch_bwd_fused(const AttnProblem& p, const CUtensorMap* tm,
 cudaError_t launch_attn_bwd_tc(const AttnProblem& p, const void* q, const void* k, const void* v, const void* o,
                                const float* lse, const void* dout, const int32_t* row_ptr, const int32_t* col_idx,
                                const int32_t* col_ptr_t, const int32_t* row_idx_t, void* dq, void* dk, void* dv,
-                               void* ws, int32_t* status, uint64_t timeout_ns, int sms, cudaStream_t stream) {
+                               void* ws, size_t ws_bytes, int32_t* status, uint64_t timeout_ns, int sms,
+                               cudaStream_t stream) {
   (void)row_ptr;
   (void)col_idx;  // the fused kernel walks the transposed lists only
   const int nt = (int)((p.N + kTile - 1) / kTile);  // 128-row tiles
@@ -709,13 +804,21 @@ cudaError_t launch_attn_bwd_tc(const AttnProblem& p, const void* q, const void* 
   float* dsum = lse2 + (size_t)p.H * Np;
   float* dq_acc = dsum + (size_t)p.H * Np;
   int32_t* item_counter = reinterpret_cast<int32_t*>(dq_acc + (size_t)p.H * Np * p.d);
-  // one clear for the dQ accumulator and the item counter right after it
-  cudaError_t e = cudaMemsetAsync(dq_acc, 0, (size_t)p.H * Np * p.d * sizeof(float) + 16, stream);
-  if (e != cudaSuccess) return e;
-  bwd_pre_kernel<<<(unsigned)((Np + 7) / 8), 256, 0, stream>>>(
+  OrderParams op{};
+  op.ptr = col_ptr_t;
+  op.order = ws_bytes >= attn_bwd_tc_ws_ordered(p) ? item_counter + 4 : nullptr;
+  op.counter = item_counter;
+  op.H = p.H;
+  op.nt = nt;
+  op.nk_fine = p.nk;
+  op.k_rows_per_tile = p.block_k == 64 ? 2 : 1;
+  const int64_t per_group = kOrderGroupBytes / (8 * Np * p.d);
+  op.heads_per_group = (int)(per_group < 1 ? 1 : (per_group > p.H ? p.H : per_group));
+  op.groups = op.order ? (p.H + op.heads_per_group - 1) / op.heads_per_group : 0;
+  bwd_pre_kernel<<<(unsigned)((Np + 7) / 8 + op.groups), 256, 0, stream>>>(
       static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(dout), lse, p.N, Np, p.H, p.d,
-      p.row_stride, lse2, dsum);
-  e = cudaGetLastError();
+      p.row_stride, lse2, dsum, dq_acc, op);
+  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // 0: 128-row blocks on both sides; 1: 128-row query blocks, 64-row key
   // blocks (merged lists); 2: 64-row query blocks, 128-row key blocks, paired
@@ -742,12 +845,13 @@ cudaError_t launch_attn_bwd_tc(const AttnProblem& p, const void* q, const void* 
   a.nq = nt;
   a.n_items = p.H * nt;
   a.nk_fine = p.nk;
-  a.k_rows_per_tile = p.block_k == 64 ? 2 : 1;
+  a.k_rows_per_tile = op.k_rows_per_tile;
   a.list_shift = p.block == 64 ? 1 : 0;
   a.scale = p.scale;
   a.scale_log2 = p.scale * 1.4426950408889634f;
   a.timeout_ns = timeout_ns;
   a.item_counter = item_counter;
+  a.order = op.order;
   __nv_bfloat16* dqb = static_cast<__nv_bfloat16*>(dq);
 #define UT_BWD_LAUNCH(DD, MM) launch_bwd_fused<DD, MM>(p, tm, a, dq_acc, dqb, sms, stream)
 #define UT_BWD_MODES(DD)                                                                    \

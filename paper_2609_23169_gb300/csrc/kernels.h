@@ -75,11 +75,13 @@ cudaError_t launch_attn_fwd_tc(const AttnProblem& p, const void* q, const void* 
                                uint64_t timeout_ns, int sms, cudaStream_t stream);
 
 // attn_bwd_tc.cu (bf16 tcgen05 backward: preprocess, fused dK/dV/dQ, dQ finalize)
-size_t attn_bwd_tc_ws(const AttnProblem& p);
+size_t attn_bwd_tc_ws(const AttnProblem& p);          // the least a call needs
+size_t attn_bwd_tc_ws_ordered(const AttnProblem& p);  // with room for the item order
 cudaError_t launch_attn_bwd_tc(const AttnProblem& p, const void* q, const void* k, const void* v, const void* o,
                                const float* lse, const void* dout, const int32_t* row_ptr, const int32_t* col_idx,
                                const int32_t* col_ptr_t, const int32_t* row_idx_t, void* dq, void* dk, void* dv,
-                               void* ws, int32_t* status, uint64_t timeout_ns, int sms, cudaStream_t stream);
+                               void* ws, size_t ws_bytes, int32_t* status, uint64_t timeout_ns, int sms,
+                               cudaStream_t stream);
 
 // tensor maps (api.cu)
 bool encode_tmap_2d_bf16(CUtensorMap* map, const void* base, uint64_t inner_elems, uint64_t rows,

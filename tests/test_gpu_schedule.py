@@ -1,0 +1,71 @@
+"""GPU parity of the attention kernels' schedules: lists of very unequal length
+(the backward's longest-first order) and a backward workspace without room for
+that order."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+from gpu_util import assert_bf16_close, bits, need_gpu, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    need_gpu()
+
+
+def _lists(bm):
+    """CSR of a [H, rows, columns] bitmap on the device."""
+    ptr = np.concatenate([[0], np.cumsum(bm.reshape(-1, bm.shape[2]).sum(1, dtype=np.int64))]).astype(np.int32)
+    return torch.from_numpy(ptr).cuda(), torch.from_numpy(np.nonzero(bm)[2].astype(np.int32)).cuda()
+
+
+def _problem(N, H, d, bq, bk, lengths, seed):
+    g = np.random.Generator(np.random.PCG64([78, seed]))
+    x = [torch.from_numpy(g.standard_normal((N, H, d)).astype(np.float32)).to(torch.bfloat16).cuda() for _ in range(4)]
+    nq, nk = -(-N // bq), -(-N // bk)
+    bm = np.zeros((H, nq, nk), dtype=np.uint8)
+    for h in range(H):
+        for i in range(nq):
+            n = min(nk, lengths[(h * nq + i) % len(lengths)])
+            bm[h, i, g.choice(nk, size=n, replace=False)] = 1
+    return x, bm
+
+
+@pytest.mark.parametrize("d,bq,bk", [(128, 128, 128), (64, 64, 64)])
+def test_backward_order_and_workspace(d, bq, bk):
+    """The item order changes nothing but the order in which dQ is summed; a
+    workspace without room for it (the size that one version of the library
+    asked for) still works."""
+    from paper_2609_23169_gb300 import ultratex as u
+    N, H = 2100, 7
+    x, bm = _problem(N, H, d, bq, bk, (1, 30, 2, 0, 9, 1), 2)
+    csr, csc = _lists(bm), _lists(np.ascontiguousarray(bm.transpose(0, 2, 1)))
+    st = u.status_word()
+    o, lse = u.ut_bsattn_fwd(*x[:3], *csr, bq, status=st, block_k=bk)
+    Np = -(-N // 128) * 128
+    least = 2 * H * Np * 4 + H * Np * d * 4 + 16
+    shape = u.attn_shape(x[0], bq, bk)
+    full = u.lib().ut_bsattn_bwd_workspace_size(ctypes.byref(shape))
+    assert full >= least + 4 * H * (Np // 128)
+    out = []
+    for size in (full, least, least + 4 * H * (Np // 128) - 1):
+        ws = torch.full((size,), 0xA5, dtype=torch.uint8, device="cuda")
+        g = u.ut_bsattn_bwd(x[0], x[1], x[2], o, lse, x[3], *csr, *csc, bq, ws=ws, status=st, block_k=bk)
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0
+        out.append(g)
+    for g in out[1:]:
+        assert_bf16_close(to_np(g[0]), to_np(out[0][0]), "dQ")
+        assert np.array_equal(bits(g[1]), bits(out[0][1])) and np.array_equal(bits(g[2]), bits(out[0][2]))
+    q, k, v = (t.double().requires_grad_(True) for t in x[:3])
+    keep = torch.from_numpy(np.repeat(np.repeat(bm, bq, 1), bk, 2)[:, :N, :N]).cuda().bool()
+    s = (torch.einsum("nhd,mhd->hnm", q, k) * d ** -0.5).masked_fill(~keep, -float("inf"))
+    seen = keep.any(2)[:, :, None]
+    p = torch.softmax(s.masked_fill(~seen, 0.0), 2) * seen
+    torch.einsum("hnm,mhd->nhd", p, v).backward(x[3].double())
+    for got, ref, name in zip(out[0], (q.grad, k.grad, v.grad), ("dQ", "dK", "dV")):
+        assert_bf16_close(to_np(got), ref.cpu().numpy(), name)
