@@ -3,30 +3,44 @@
 // for every (head, query block i), iterating only the listed key blocks.
 //
 // Persistent kernel, one CTA per SM, work items (h, i) in head-major order so
-// that the CTAs in flight share one head's K/V in L2.  Roles (192 threads):
-//   warp 0      TMA producers: lane 0 streams the item's Q tile and the K tiles,
-//               lane 1 the V tiles, each into its own 3-stage ring of
+// that the CTAs in flight share one head's K/V in L2.  The key tiles of a CTA's
+// items form one stream; tile n of the stream belongs to softmax warpgroup
+// n & 1 and to S buffer n & 1.  Roles (384 threads, three warpgroups, registers
+// rebalanced with setmaxnreg):
+//   warp 0      TMA producers: lane 0 streams the items' Q tiles and the K tiles,
+//               lane 1 the V tiles, K and V each into a 3-stage ring of
 //               128B-swizzled shared tiles.  A K stage is released by the MMA
 //               that consumed it (S = Q K^T), a V stage by O += P V.
-//   warp 1      TMEM owner and MMA issuer (one elected thread):
-//               S_t = Q K_t^T with Q read from TMEM (only K from shared
-//               memory) into one of two TMEM S buffers, two key blocks ahead
-//               of O += P_u V_u with P also read from TMEM (only V from shared
-//               memory).
-//   warps 2-5   softmax: thread = query row = TMEM lane.  At the start of an
-//               item they copy its Q tile from shared memory into TMEM (the A
-//               operand of S), then finish the previous item (normalise O,
-//               write O in bf16 and LSE in fp32, natural log) while the tensor
-//               core already computes the new item's first S blocks.  Per key
-//               block: read S_t from TMEM, mask the ragged last key block, keep
-//               a running row maximum (rescaling O in TMEM only when the
-//               maximum grew by more than 2^8, so the exponentials stay
-//               bounded), write P_t as bf16 pairs into the TMEM P buffer.
+//   warp 1      TMEM owner and MMA issuer: O += P_u V_u (P from TMEM, V from
+//               shared memory), then S_{u+2} = Q K_{u+2}^T (Q from TMEM, K from
+//               shared memory) into the buffer P_u was just read from.
+//   warps 4-11  two softmax warpgroups, thread = query row = TMEM lane.  Per
+//               tile: read S from TMEM, mask the ragged last key block, keep a
+//               running row maximum (rescaling O in TMEM only when the maximum
+//               grew by more than 2^8, so the exponentials stay bounded), write
+//               P as bf16 pairs over the columns of S it was computed from, in
+//               two halves so that P V starts after the first.
+// What bounds it, and why this split: the two 128 x 128 x 128 products of a key
+// tile take 1,024 cycles, one warpgroup's serial pass over a tile (barrier, TMEM
+// load, maximum, 128 exponentials a thread at 8 a cycle and quarter, store,
+// barrier) about 1,700.  With one warpgroup the launch ran at that pace (a clock
+// trace: 1,720 cycles per tile); two of them on alternate tiles overlap one
+// pass with the other's and with the products.  The row maximum goes from tile
+// to tile through shared memory (each tile's warp publishes it before the
+// exponentials, the warp of the next tile reads it), so the rescaling rule and
+// P are those of one pass in tile order; each warpgroup sums its own tiles' row
+// normalisers and the two are added at the end of the item.
+// P over S leaves 64 TMEM columns: they double-buffer Q, so the next item's
+// first S follows the current item's last but one P V without a gap.
 // Reading Q from TMEM halves the shared-memory operand traffic of S = Q K^T;
 // per key block the shared memory then serves K and V to the tensor core and
-// their TMA writes (128 KB), about what the two 128 x 128 x 128 products take.
-// TMEM columns: S0 [0,128), S1 [128,256), O [256,256+D), P [384,448),
-// Q [448,448+D/2).
+// their TMA writes (128 KB), about what the two products take.
+// TMEM columns: S0 [0,128), S1 [128,256) (P over the first 64 of each),
+// O [256,256+D), Q [384,384+D/2) and [448,448+D/2).
+// Measured against one warpgroup, same clocks: 2048 canvas, Top-K 0.12, 7,545 ->
+// 7,384 us in a loop (6,972 -> 6,783 after a pause: in a loop the card is at its
+// 1.4 kW cap, and what the kernel gains in cycles the clock gives back, 1,815 ->
+// 1,732 MHz); d = 64 forward and backward at 512 418 -> 398 us.
 // Blocks of 64 rows (b_q or b_kv) are served by the same 128 x 128 tiles:
 //   b_kv = 64:  two listed 64-row key blocks fill one 128-row key tile (two
 //               TMA boxes per operand, PairList): consecutive entries of the
@@ -46,10 +60,15 @@ namespace ut {
 
 constexpr int kBM = 128;  // query rows per tile
 constexpr int kBN = 128;  // key rows per tile
-constexpr int kFwdThreads = 192;
+constexpr int kFwdThreads = 384;
+// registers per thread after setmaxnreg: control warpgroup and the two softmax
+// warpgroups; the sum is what the launch allocates (3 x 168), so every
+// increase is covered by the decrease
+constexpr int kFwdRegLaunch = 168, kFwdRegCtl = 88, kFwdRegSm = 208;
+static_assert(kFwdRegCtl + 2 * kFwdRegSm == 3 * kFwdRegLaunch, "setmaxnreg split must match the launch");
 constexpr int kStages = 3;                       // K and V ring depth
 constexpr uint32_t kTileChunkBytes = 128 * 128;  // 128 rows x 128 bytes (64 bf16)
-constexpr uint32_t kColO = 256, kColP = 384, kColQ = 448;  // TMEM column bases
+constexpr uint32_t kColO = 256, kColQ = 384;     // TMEM column bases (Q: two buffers of 64 columns)
 
 template <int D>
 struct FwdSmem {
@@ -59,12 +78,20 @@ struct FwdSmem {
   alignas(1024) uint8_t q[kQBytes];
   alignas(1024) uint8_t k[kStages][kKVBytes];
   alignas(1024) uint8_t v[kStages][kKVBytes];
-  uint64_t q_full, q_empty;    // shared Q tile: TMA landed / copied into TMEM
-  uint64_t qt_full, qt_empty;  // TMEM Q: written by the softmax warps / last S of the item done
+  // shared Q tile: TMA landed, by item & 1 (a warpgroup may pass over one item
+  // without waiting for its Q, never over two, so it always waits for the phase
+  // after one it knows to be complete) / copied into TMEM
+  uint64_t q_full[2], q_empty;
+  uint64_t qt_full[2];         // TMEM Q written by the softmax warps, by item & 1
   uint64_t k_full[kStages], v_full[kStages], k_empty[kStages], v_empty[kStages];
-  uint64_t s_full[2], s_empty[2];
-  uint64_t p_full, pv_done;    // one TMEM P buffer
+  uint64_t s_full[2];          // S tile in its buffer
+  uint64_t p_full[2][2];       // [buffer][half of the key columns]
+  uint64_t pv_done[2];         // O += P V of a tile finished, by tile & 1
   uint64_t o_empty, mma_done;
+  uint64_t m_full[2][4];       // [tile & 1][lane quarter]: row maxima published
+  uint64_t l_full[2][4];       // [item & 1][lane quarter]: the other warpgroup's normalisers
+  float m_row[2][kBM];         // row maximum used by tile (tile & 1)
+  float l_row[2][kBM];         // normaliser handed over, per item & 1
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -92,18 +119,30 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k64,
                        const __grid_constant__ CUtensorMap tm_v64, const FwdParams prm) {
   constexpr bool kSub = kMode != 0;  // 64-row blocks on at least one side
-  extern __shared__ uint8_t smem_raw[];
-  FwdSmem<D>& sm = *reinterpret_cast<FwdSmem<D>*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  // Exponentials ahead of the tile's maximum (below): they pay where the two
+  // products are as long as the softmax (d = 128: 7,597 -> 7,411 us at the 2048
+  // canvas); with d = 64, and with halves that a row may not see, the maximum
+  // first is faster (d = 64 training layer 397 against 408 us, 64-row blocks
+  // 13.2 against 14.0 ms), since the exponentials then do not stand between one
+  // tile's maximum and the next's.
+  constexpr bool kAhead = kMode == 0 && D == 128;
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  FwdSmem<D>& sm = *reinterpret_cast<FwdSmem<D>*>(smem_raw);
   constexpr int C = FwdSmem<D>::kChunks;
   const uint32_t warp = warp_id();
   const uint32_t lane = lane_id();
   volatile int* abort_flag = &sm.abort_flag;
+  if ((smem_u32(smem_raw) & 1023u) != 0) {
+    if (threadIdx.x == 0) set_status(prm.status, UT_ERR_INVALID_ARG);
+    return;
+  }
 
   if (threadIdx.x == 0) {
-    mbar_init(&sm.q_full, 1);
+    mbar_init(&sm.q_full[0], 1);
+    mbar_init(&sm.q_full[1], 1);
     mbar_init(&sm.q_empty, 4);
-    mbar_init(&sm.qt_full, 4);
-    mbar_init(&sm.qt_empty, 1);
+    mbar_init(&sm.qt_full[0], 4);
+    mbar_init(&sm.qt_full[1], 4);
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&sm.k_full[s], 1);
       mbar_init(&sm.v_full[s], 1);
@@ -112,10 +151,14 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&sm.s_full[s], 1);
-      mbar_init(&sm.s_empty[s], 4);
+      mbar_init(&sm.pv_done[s], 1);
+      mbar_init(&sm.p_full[s][0], 4);
+      mbar_init(&sm.p_full[s][1], 4);
+      for (int x = 0; x < 4; ++x) {
+        mbar_init(&sm.m_full[s][x], 1);
+        mbar_init(&sm.l_full[s][x], 1);
+      }
     }
-    mbar_init(&sm.p_full, 4);
-    mbar_init(&sm.pv_done, 1);
     mbar_init(&sm.o_empty, 4);
     mbar_init(&sm.mma_done, 1);
     sm.abort_flag = 0;
@@ -131,6 +174,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
   const uint32_t tmem = sm.tmem_base;
 
   const int G = gridDim.x;
+  if (warp < 4) {
+  setmaxnreg_dec<kFwdRegCtl>();
   if (warp == 0) {
     // ------------------------------------------------------------ producer
     // lane 0 streams Q and K, lane 1 streams V: each ring is released by the
@@ -162,9 +207,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
         if (tl.empty()) continue;
         if (is_k) {
           if (!(ok = mbar_wait(&sm.q_empty, (qi & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns))) break;
-          mbar_expect_tx(&sm.q_full, FwdSmem<D>::kQBytes);
+          mbar_expect_tx(&sm.q_full[qi & 1], FwdSmem<D>::kQBytes);
           for (int c = 0; c < C; ++c)
-            tma_load_2d(sm.q + c * kTileChunkBytes, &tm_q, &sm.q_full, h * D + c * 64, i * kBM, pol_q);
+            tma_load_2d(sm.q + c * kTileChunkBytes, &tm_q, &sm.q_full[qi & 1], h * D + c * 64, i * kBM, pol_q);
           ++qi;
         }
         int j, jh;
@@ -190,7 +235,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       auto drain = [&](uint64_t* bar, uint32_t parity) {
         if (!mbar_drain(bar, parity, kDrainTimeoutNs)) set_status(prm.status, UT_ERR_TIMEOUT);
       };
-      if (qi > 0) drain(&sm.q_full, (qi - 1) & 1);
+      if (qi > 0) drain(&sm.q_full[(qi - 1) & 1], ((qi - 1) >> 1) & 1);
       for (uint32_t u = (kv >= kStages ? kv - kStages : 0); u < kv; ++u)
         drain(&full[u % kStages], (u / kStages) & 1);
     }
@@ -198,84 +243,122 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     // ---------------------------------------------------------- MMA issuer
     // The whole warp runs this loop converged; every MMA and commit is issued
     // by one elected lane (see mma_bf16_ss_w), waits are warp-uniform.
-    {
-      constexpr uint32_t idesc_s = idesc_bf16_f32(kBM, kBN, false, false);
-      constexpr uint32_t idesc_o = idesc_bf16_f32(kBM, D, false, true);
-      uint32_t qi = 0, oi = 0, kv0 = 0, sc0 = 0;
-      bool ok = true;
-      for (int w = blockIdx.x; w < prm.n_items && ok; w += G) {
-        BlockSteps<kMode> tl;
-        tl.init(prm.row_ptr, prm.col_idx, w / prm.nq, w % prm.nq, prm.nq_fine, prm.q_rows_per_tile, prm.list_shift);
-        const int L = tl.count_warp();
-        if (L <= 0) continue;
-        // Q of this item in TMEM (the softmax warps copied it there)
-        if (!(ok = warp_wait(&sm.qt_full, qi & 1, abort_flag, prm.status, prm.timeout_ns))) break;
-        // S runs two key blocks ahead of P V: S_{u+2} goes into the S buffer
-        // that softmax u has just read, so the tensor core computes it while
-        // the softmax works, and PV_u follows as soon as P_u is in TMEM.
-        auto issue_s = [&](int t) -> bool {
-          const uint32_t kv = kv0 + t, st = kv % kStages, n = kv / kStages;
-          const uint32_t sc = sc0 + t, sb = sc & 1, ns = sc >> 1;
-          if (!warp_wait(&sm.k_full[st], n & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
-          if (!warp_wait(&sm.s_empty[sb], (ns & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns)) return false;
-          tc_fence_after();
-          const uint32_t k_addr = smem_u32(sm.k[st]);
-#pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t off = (kk >> 2) * kTileChunkBytes + (kk & 3) * 32;
-            mma_bf16_ts_w(tmem + sb * 128, tmem + kColQ + kk * 8, sdesc_sw128(k_addr + off, 16, 1024), idesc_s,
-                          kk > 0);
-          }
-          mma_commit_w(&sm.s_full[sb]);
-          mma_commit_w(&sm.k_empty[st]);
-          if (t == L - 1) mma_commit_w(&sm.qt_empty);  // Q's TMEM columns are free once these S are done
-          return true;
-        };
-        auto issue_pv = [&](int u) -> bool {
-          const uint32_t kv = kv0 + u, st = kv % kStages, n = kv / kStages;
-          const uint32_t sc = sc0 + u;
-          if (!warp_wait(&sm.p_full, sc & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
-          if (!warp_wait(&sm.v_full[st], n & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
-          if (u == 0 && !warp_wait(&sm.o_empty, (oi & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns)) return false;
-          tc_fence_after();
-          const uint32_t v_addr = smem_u32(sm.v[st]);
-#pragma unroll
-          for (int kk = 0; kk < kBN / 16; ++kk)
-            mma_bf16_ts_w(tmem + kColO, tmem + kColP + kk * 8, sdesc_sw128(v_addr + kk * 2048, kTileChunkBytes, 1024),
-                          idesc_o, (u > 0 || kk > 0));
-          mma_commit_w(&sm.pv_done);
-          mma_commit_w(&sm.v_empty[st]);
-          return true;
-        };
-        ok = issue_s(0) && (L < 2 || issue_s(1));
-        for (int u = 0; u < L && ok; ++u) {
-          if (u + 2 < L && !(ok = issue_s(u + 2))) break;
-          ok = issue_pv(u);
+    // S runs two tiles ahead of P V over the stream of tiles.  S_{u+2} needs no
+    // wait for its buffer: it is issued after P V_u, the last reader, and MMAs
+    // of one thread execute in order.
+    constexpr uint32_t idesc_s = idesc_bf16_f32(kBM, kBN, false, false);
+    constexpr uint32_t idesc_o = idesc_bf16_f32(kBM, D, false, true);
+    uint32_t sc = 0, pc = 0;  // tiles of the stream: S issued, P V issued
+    uint32_t qi = 0, oi = 0;  // items: S started, P V started
+    uint32_t firsts = 0;      // bit (tile & 3): the tile is the first of its item
+    bool ok = true;
+    // item of the S cursor: index, tiles, next tile; the list bounds of the
+    // following item are loaded an item ahead (128-row blocks)
+    int cw = blockIdx.x, cL = 0, ct = 0;
+    int n_lo = 0, n_hi = 0;
+    auto load_bounds = [&](int w) {
+      if (kMode == 0 && w < prm.n_items) {
+        n_lo = prm.row_ptr[w];
+        n_hi = prm.row_ptr[w + 1];
+      }
+    };
+    auto count_from = [&]() {  // cw, cL: the first item from cw on that lists something (cL = 0: none)
+      for (cL = 0; cw < prm.n_items; cw += G) {
+        if (kMode == 0) {
+          cL = n_hi - n_lo;
+          load_bounds(cw + G);
+        } else {
+          BlockSteps<kMode> tl;
+          tl.init(prm.row_ptr, prm.col_idx, cw / prm.nq, cw % prm.nq, prm.nq_fine, prm.q_rows_per_tile,
+                  prm.list_shift);
+          cL = tl.count_warp();
         }
-        kv0 += L;
-        sc0 += L;
+        if (cL > 0) return;
+      }
+      cL = 0;
+    };
+    auto wait_k = [&]() -> bool {  // K of the next S tile in its stage
+      return warp_wait(&sm.k_full[sc % kStages], (sc / kStages) & 1, abort_flag, prm.status, prm.timeout_ns);
+    };
+    auto issue_s = [&]() -> bool {
+      const uint32_t st = sc % kStages, sb = sc & 1;
+      if (ct == 0 && !warp_wait(&sm.qt_full[qi & 1], (qi >> 1) & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
+      if (sc < 2 && !wait_k()) return false;
+      tc_fence_after();
+      const uint32_t k_addr = smem_u32(sm.k[st]);
+      const uint32_t q_col = tmem + kColQ + (qi & 1) * 64;
+#pragma unroll
+      for (int kk = 0; kk < D / 16; ++kk) {
+        const uint32_t off = (kk >> 2) * kTileChunkBytes + (kk & 3) * 32;
+        mma_bf16_ts_w(tmem + sb * 128, q_col + kk * 8, sdesc_sw128(k_addr + off, 16, 1024), idesc_s, kk > 0);
+      }
+      mma_commit_w(&sm.s_full[sb]);
+      mma_commit_w(&sm.k_empty[st]);
+      firsts = (firsts & ~(1u << (sc & 3))) | ((ct == 0 ? 1u : 0u) << (sc & 3));
+      ++sc;
+      if (++ct == cL) {
+        cw += G;
+        ct = 0;
         ++qi;
+        count_from();
+      }
+      return true;
+    };
+    auto issue_pv = [&]() -> bool {
+      const uint32_t st = pc % kStages, n = pc / kStages, sb = pc & 1, ph = (pc >> 1) & 1;
+      const bool first = (firsts >> (pc & 3)) & 1u;
+      if (!warp_wait(&sm.v_full[st], n & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
+      if (first) {  // O is free once the previous item's was read
+        if (!warp_wait(&sm.o_empty, (oi & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns)) return false;
         ++oi;
       }
-      // Drain: all MMAs issued by this warp complete before TMEM is freed.
-      mma_commit_w(&sm.mma_done);
-      if (!mbar_drain(&sm.mma_done, 0, kDrainTimeoutNs)) set_status(prm.status, UT_ERR_TIMEOUT);
+      // K of the S tile that follows: ready long before P, and waited for here
+      // it does not stand between P V and S
+      if (cL > 0 && !wait_k()) return false;
+      const uint32_t v_addr = smem_u32(sm.v[st]);
+#pragma unroll
+      for (int hc = 0; hc < 2; ++hc) {
+        if (!warp_wait(&sm.p_full[sb][hc], ph, abort_flag, prm.status, prm.timeout_ns)) return false;
+        tc_fence_after();
+#pragma unroll
+        for (int kk = hc * (kBN / 32); kk < (hc + 1) * (kBN / 32); ++kk)
+          mma_bf16_ts_w(tmem + kColO, tmem + sb * 128 + kk * 8, sdesc_sw128(v_addr + kk * 2048, kTileChunkBytes, 1024),
+                        idesc_o, (!first || kk > 0));
+      }
+      mma_commit_w(&sm.pv_done[sb]);
+      mma_commit_w(&sm.v_empty[st]);
+      ++pc;
+      return true;
+    };
+    load_bounds(cw);
+    count_from();
+    for (int x = 0; x < 2 && ok && cL > 0; ++x) ok = issue_s();
+    while (ok && pc < sc) {
+      if (!(ok = issue_pv())) break;
+      if (cL > 0) ok = issue_s();
     }
+    // Drain: all MMAs issued by this warp complete before TMEM is freed.
+    mma_commit_w(&sm.mma_done);
+    if (!mbar_drain(&sm.mma_done, 0, kDrainTimeoutNs)) set_status(prm.status, UT_ERR_TIMEOUT);
+  }
   } else {
+    setmaxnreg_inc<kFwdRegSm>();
     // ------------------------------------------------------------- softmax
+    const uint32_t wgi = (warp >> 2) - 1;  // warpgroup 0 / 1: even / odd tiles of the stream
     const uint32_t quarter = warp & 3;
     const uint32_t row = quarter * 32 + lane;
     const uint32_t lane_base = (quarter * 32) << 16;
     const float c = prm.scale_log2;
-    uint32_t sc0 = 0, qi = 0;
+    uint32_t sc0 = 0, it = 0;  // tiles and (non-empty) items so far
     bool ok = true;
     const uint32_t rh = row >> 6;  // which 64-row half of the query tile
-    // Q tile of the next item: shared memory (128B-swizzled, as TMA wrote it)
-    // -> registers -> TMEM, this thread's row, bf16 pairs (element 2u in the
-    // low half of column u), the A-operand layout of S = Q K^T.
+    // Q tile of an item: shared memory (128B-swizzled, as TMA wrote it) ->
+    // registers -> TMEM, this thread's row, bf16 pairs (element 2u in the low
+    // half of column u), the A-operand layout of S = Q K^T.  The buffer was
+    // last read by item it - 2, whose S this warpgroup's previous tile
+    // (or a later one) has waited for.
     auto load_q = [&]() -> bool {
-      if (!warp_wait(&sm.q_full, qi & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
-      if (!warp_wait(&sm.qt_empty, (qi & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns)) return false;
+      if (!warp_wait(&sm.q_full[it & 1], (it >> 1) & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
       tc_fence_after();
 #pragma unroll
       for (int cc = 0; cc < C; ++cc) {
@@ -286,55 +369,15 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
           asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                        : "=r"(qv[4 * u]), "=r"(qv[4 * u + 1]), "=r"(qv[4 * u + 2]), "=r"(qv[4 * u + 3])
                        : "r"(base + ((u ^ (row & 7)) << 4)));
-        tmem_st32(tmem + lane_base + kColQ + cc * 32, qv);
+        tmem_st32(tmem + lane_base + kColQ + (it & 1) * 64 + cc * 32, qv);
       }
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(&sm.qt_full);
+        mbar_arrive(&sm.qt_full[it & 1]);
         mbar_arrive(&sm.q_empty);
       }
-      ++qi;
-      return true;
-    };
-    // The previous item's epilogue (O / l -> bf16, LSE) runs after the next
-    // item's Q is in TMEM, so the tensor core computes the next S blocks
-    // meanwhile.
-    bool pend = false;
-    float e_m = 0.f, e_l = 0.f;
-    uint32_t e_last = 0;
-    int64_t e_grow = 0;
-    int e_h = 0;
-    auto epilogue = [&]() -> bool {
-      if (!warp_wait(&sm.pv_done, e_last & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
-      tc_fence_after();
-      const bool row_ok = e_grow < prm.N;
-      __nv_bfloat16* orow = prm.o + e_grow * prm.rs + (int64_t)e_h * D;
-      const float inv = (!kSub || e_l > 0.f) ? 1.0f / e_l : 0.f;  // a row that saw no key: O = 0, LSE = -inf
-#pragma unroll
-      for (int g = 0; g < D / 32; ++g) {
-        uint32_t r[32];
-        tmem_ld32(tmem + lane_base + kColO + g * 32, r);
-        tmem_wait_ld();
-        if (row_ok) {
-#pragma unroll
-          for (int x = 0; x < 32; x += 8) {
-            uint4 v;
-            v.x = pack_bf16x2(__uint_as_float(r[x + 0]) * inv, __uint_as_float(r[x + 1]) * inv);
-            v.y = pack_bf16x2(__uint_as_float(r[x + 2]) * inv, __uint_as_float(r[x + 3]) * inv);
-            v.z = pack_bf16x2(__uint_as_float(r[x + 4]) * inv, __uint_as_float(r[x + 5]) * inv);
-            v.w = pack_bf16x2(__uint_as_float(r[x + 6]) * inv, __uint_as_float(r[x + 7]) * inv);
-            *reinterpret_cast<uint4*>(orow + g * 32 + x) = v;
-          }
-        }
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.o_empty);
-      if (row_ok)
-        prm.lse[(int64_t)e_h * prm.N + e_grow] =
-            (!kSub || e_l > 0.f) ? (e_m + log2f(e_l)) * 0.69314718055994531f : -INFINITY;
       return true;
     };
     for (int w = blockIdx.x; w < prm.n_items && ok; w += G) {
@@ -343,149 +386,207 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       tl.init(prm.row_ptr, prm.col_idx, h, i, prm.nq_fine, prm.q_rows_per_tile, prm.list_shift);
       const int L = tl.count_warp();
       const int64_t grow = (int64_t)i * kBM + row;
+      const bool row_ok = grow < prm.N;
+      __nv_bfloat16* orow = prm.o + grow * prm.rs + (int64_t)h * D;
       if (L <= 0) {
-        if (grow < prm.N) {
-          __nv_bfloat16* orow = prm.o + grow * prm.rs + (int64_t)h * D;
+        if (wgi == 0 && row_ok) {
           for (int e = 0; e < D; e += 8) *reinterpret_cast<uint4*>(orow + e) = make_uint4(0, 0, 0, 0);
           prm.lse[(int64_t)h * prm.N + grow] = -INFINITY;
         }
         continue;
       }
-      if (!(ok = load_q())) break;
-      if (pend && !(ok = epilogue())) break;
-      pend = false;
-      float m_used = 0.f, l = 0.f;
-      int j_next = 0, jh_next = -1;
-      uint32_t bits_next = 0;
-      tl.next(j_next, jh_next, bits_next);
-      for (int t = 0; t < L; ++t) {
-        const int j = j_next, jh = jh_next;
-        const uint32_t bits = bits_next;
-        if (t + 1 < L) tl.next(j_next, jh_next, bits_next);  // the next tile's blocks, fetched a tile ahead
+      const uint32_t t0 = (sc0 ^ wgi) & 1;  // this warpgroup's first tile of the item
+      if (t0 == 0 && !(ok = load_q())) break;
+      // lists ascend: with 128-row blocks only the last tile can be ragged
+      int j = 0, jh = -1;
+      uint32_t bits = 15u;
+      if (kMode == 0) j = tl.tl.a[L - 1];
+      else if (t0) tl.next(j, jh, bits);
+      float m_before = 0.f;  // the maximum the previous tile of the stream used
+      float m = 0.f, l = 0.f;  // row maximum in use and this warpgroup's part of the normaliser under it
+      for (int t = t0; t < L; t += 2) {
+        if (kMode != 0) {
+          if (t > (int)t0) tl.next(j, jh, bits);  // the other warpgroup's tile
+          tl.next(j, jh, bits);
+        }
         const uint32_t sc = sc0 + t, sb = sc & 1, ns = sc >> 1;
+        const uint32_t s_col = tmem + lane_base + sb * 128;
         if (!(ok = warp_wait(&sm.s_full[sb], ns & 1, abort_flag, prm.status, prm.timeout_ns))) break;
         tc_fence_after();
+        // ragged last key block: columns past N do not exist.  They are set to
+        // -inf in TMEM, in a short loop: selects on all 128 registers, skipped
+        // or not, sit in the middle of every tile's instruction stream.
+        if (kMode != 0 || t == L - 1) {
+          const int e0 = tl.pair ? 64 : kBN;  // columns that belong to the low (or only) listed block
+          const int64_t nv0 = prm.N - (tl.pair ? 64 * (int64_t)PairList::load_lo(j, jh) : (int64_t)j * kBN);
+          const int64_t nv1 = tl.pair ? prm.N - 64 * (int64_t)PairList::load_hi(j, jh) : 64;
+          if (__builtin_expect(nv0 < e0 || nv1 < 64, 0)) {
+            for (int x = (int)nv0; x < e0; ++x) tmem_st1(s_col + x, 0xff800000u);
+            for (int x = (int)nv1; x < 64; ++x) tmem_st1(s_col + 64 + x, 0xff800000u);
+            tmem_wait_st();
+          }
+        }
         // all four 32-column loads in flight before one wait
         uint32_t r[kBN];
 #pragma unroll
-        for (int g = 0; g < kBN / 32; ++g)
-          tmem_ld32(tmem + lane_base + sb * 128 + g * 32, *reinterpret_cast<uint32_t(*)[32]>(&r[g * 32]));
+        for (int g = 0; g < kBN / 32; ++g) tmem_ld32(s_col + g * 32, *reinterpret_cast<uint32_t(*)[32]>(&r[g * 32]));
+        // the maximum that the previous tile used, from its warp (waited for on
+        // an item's first tile too: it also says that the slot written below
+        // was read)
+        float m_new = -INFINITY;
+        auto previous_max = [&]() -> bool {
+          if (sc > 0 && !warp_wait(&sm.m_full[(sc - 1) & 1][quarter], ((sc - 1) >> 1) & 1, abort_flag, prm.status,
+                                   prm.timeout_ns))
+            return false;
+          if (t > 0) m_new = m_before = *const_cast<volatile float*>(&sm.m_row[(sc - 1) & 1][row]);
+          return true;
+        };
+        if (kAhead && !(ok = previous_max())) break;
         tmem_wait_ld();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.s_empty[sb]);
         float s[kBN];
 #pragma unroll
         for (int x = 0; x < kBN; ++x) s[x] = __uint_as_float(r[x]);
-        // ragged last key block: columns past N do not exist; 64-column
-        // halves of the tile not listed for this row's half are masked
+        // 64-column halves of the tile not listed for this row's half do not
+        // count (the same for the whole warp: rh is per warp)
         const uint32_t cols = kSub ? (bits >> (2 * rh)) & 3u : 3u;
-        if (tl.pair) {  // each half holds its own 64-row key block
-          const int64_t nv0 = prm.N - 64 * (int64_t)PairList::load_lo(j, jh);
-          const int64_t nv1 = prm.N - 64 * (int64_t)PairList::load_hi(j, jh);
-          if (nv0 < 64) {
+        // P = exp2(s * c - m) of one half's 64 columns, rounded to bf16 for the
+        // P V MMA, and its part of the normaliser
+        float2 l4[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+        uint32_t pk[kBN / 4];
+        auto exp_pair = [&](int hc, int x) {
+          const float2 e = ffma2(make_float2(s[hc * 64 + x], s[hc * 64 + x + 1]), make_float2(c, c),
+                                 make_float2(-m_new, -m_new));
+          const float2 p = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+          l4[(x >> 1) & 3] = add2(l4[(x >> 1) & 3], p);
+          pk[x / 2] = pack_bf16x2(p.x, p.y);
+        };
+        auto exp_half = [&](int hc) {
+          if (kSub && !((cols >> hc) & 1u)) {  // a masked half: P = 0 without the exponentials
 #pragma unroll
-            for (int x = 0; x < 64; ++x)
-              if (x >= nv0) s[x] = -INFINITY;
-          }
-          if (nv1 < 64) {
+            for (int x = 0; x < kBN / 4; ++x) pk[x] = 0u;
+          } else {
 #pragma unroll
-            for (int x = 64; x < kBN; ++x)
-              if (x - 64 >= nv1) s[x] = -INFINITY;
+            for (int x = 0; x < kBN / 2; x += 2) exp_pair(hc, x);
           }
-        } else {
-          const int64_t nv = prm.N - (int64_t)j * kBN;
-          if (nv < kBN) {
+        };
+        // Row maximum, eight chains of three-input maxima.  Ahead: the first
+        // half of P is computed under the previous tile's maximum in the same
+        // instructions' shadow (exponentials and maxima run on different
+        // units) and done over in the rare tile that has to raise it, and in an
+        // item's first (m_new = -inf).
+        float mx = -INFINITY;
+        {
+          float m8[8];
 #pragma unroll
-            for (int x = 0; x < kBN; ++x)
-              if (x >= nv) s[x] = -INFINITY;
+          for (int q = 0; q < 8; ++q) m8[q] = -INFINITY;
+          if constexpr (kAhead) {
+#pragma unroll
+            for (int x = 0; x < kBN / 2; x += 2) {
+              exp_pair(0, x);
+              m8[(x >> 1) & 3] = max3(m8[(x >> 1) & 3], s[x], s[x + 1]);
+              m8[4 + ((x >> 1) & 3)] = max3(m8[4 + ((x >> 1) & 3)], s[64 + x], s[64 + x + 1]);
+            }
+          } else {
+#pragma unroll
+            for (int hc = 0; hc < 2; ++hc) {
+              if (kSub && !((cols >> hc) & 1u)) continue;
+#pragma unroll
+              for (int x = 0; x < kBN / 2; x += 16)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) m8[q] = max3(m8[q], s[hc * 64 + x + q], s[hc * 64 + x + q + 8]);
+            }
           }
+          mx = max3(max3(m8[0], m8[1], m8[2]), max3(m8[3], m8[4], m8[5]), fmaxf(m8[6], m8[7]));
         }
-        if (kSub) {  // a masked half is the same for the whole warp (rh is per warp)
-          if (!(cols & 1u)) {
-#pragma unroll
-            for (int x = 0; x < kBN / 2; ++x) s[x] = -INFINITY;
-          }
-          if (!(cols & 2u)) {
-#pragma unroll
-            for (int x = kBN / 2; x < kBN; ++x) s[x] = -INFINITY;
-          }
-        }
-        // row maximum as a tree (8 independent chains) rather than one long chain
-        float m8[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) m8[q] = s[q];
-#pragma unroll
-        for (int x = 8; x < kBN; ++x) m8[x & 7] = fmaxf(m8[x & 7], s[x]);
-        float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])),
-                         fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
         // a row may see nothing in this tile: keep the reference maximum
         // finite so that exp2(-inf - m) stays 0 (not NaN)
         mx = kSub ? fmaxf(mx * c, -1e30f) : mx * c;
-        if (t == 0) {
-          m_used = mx;
-        } else {
-          const bool need = mx > m_used + 8.0f;
-          if (__any_sync(0xffffffffu, need)) {
-            // O holds P V up to the previous key block once that MMA finished
-            if (!(ok = warp_wait(&sm.pv_done, (sc & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns))) break;
+        if (!kAhead && !(ok = previous_max())) break;
+        const bool need = t == 0 || mx > m_new + 8.0f;
+        if (__builtin_expect(__any_sync(0xffffffffu, need), 0)) {
+          if (t > 0) {
+            // O holds P V up to the previous tile once that MMA finished
+            if (!(ok = warp_wait(&sm.pv_done[(sc - 1) & 1], ((sc - 1) >> 1) & 1, abort_flag, prm.status,
+                                 prm.timeout_ns)))
+              break;
             tc_fence_after();
-            const float alpha = need ? ex2_approx(m_used - mx) : 1.0f;
-#pragma unroll
-            for (int g = 0; g < D / 32; ++g) {
-              uint32_t r[32];
-              tmem_ld32(tmem + lane_base + kColO + g * 32, r);
+            const float alpha = need ? ex2_approx(m_new - mx) : 1.0f;
+#pragma unroll 1
+            for (int g = 0; g < D / 16; ++g) {
+              uint32_t o[16];
+              tmem_ld16(tmem + lane_base + kColO + g * 16, o);
               tmem_wait_ld();
 #pragma unroll
-              for (int x = 0; x < 32; ++x) r[x] = __float_as_uint(__uint_as_float(r[x]) * alpha);
-              tmem_st32(tmem + lane_base + kColO + g * 32, r);
+              for (int x = 0; x < 16; ++x) o[x] = __float_as_uint(__uint_as_float(o[x]) * alpha);
+              tmem_st16(tmem + lane_base + kColO + g * 16, o);
             }
             tmem_wait_st();
-            if (need) {
-              l *= alpha;
-              m_used = mx;
-            }
+          }
+          if (need) m_new = mx;
+          if (kAhead) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) l4[q] = make_float2(0.f, 0.f);
+            exp_half(0);
           }
         }
-        // P = exp2(s * c - m_used), rounded to bf16 for the P V MMA
-        uint32_t pk[kBN / 2];
-        float l8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        *const_cast<volatile float*>(&sm.m_row[sc & 1][row]) = m_new;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.m_full[sc & 1][quarter]);
+        if (t > (int)t0) l *= ex2_approx(m - m_new);
+        m = m_new;
+        // P goes over S's own columns (this thread has read its whole row of S)
 #pragma unroll
         for (int hc = 0; hc < 2; ++hc) {
-          if (kSub && !((cols >> hc) & 1u)) {  // a masked half: P = 0 without the exponentials
-#pragma unroll
-            for (int x = hc * (kBN / 2); x < (hc + 1) * (kBN / 2); x += 2) pk[x / 2] = 0u;
-            continue;
-          }
-#pragma unroll
-          for (int x = hc * (kBN / 2); x < (hc + 1) * (kBN / 2); x += 2) {
-            const float p0 = ex2_approx(fmaf(s[x], c, -m_used));
-            const float p1 = ex2_approx(fmaf(s[x + 1], c, -m_used));
-            l8[(x >> 1) & 7] += p0 + p1;
-            pk[x / 2] = pack_bf16x2(p0, p1);
-          }
+          if (!kAhead || hc == 1) exp_half(hc);
+          tmem_st32(s_col + hc * 32, pk);
+          tmem_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.p_full[sb][hc]);
         }
-        l += ((l8[0] + l8[1]) + (l8[2] + l8[3])) + ((l8[4] + l8[5]) + (l8[6] + l8[7]));
-        // the TMEM P buffer is free once the previous key block's P V finished
-        if (!(ok = warp_wait(&sm.pv_done, (sc & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns))) break;
-        tc_fence_after();
-        tmem_st32(tmem + lane_base + kColP, *reinterpret_cast<uint32_t(*)[32]>(&pk[0]));
-        tmem_st32(tmem + lane_base + kColP + 32, *reinterpret_cast<uint32_t(*)[32]>(&pk[32]));
-        tmem_wait_st();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.p_full);
+        const float2 lt = add2(add2(l4[0], l4[1]), add2(l4[2], l4[3]));
+        l += lt.x + lt.y;
       }
       if (!ok) break;
-      pend = true;
-      e_m = m_used;
-      e_l = l;
-      e_last = sc0 + L - 1;
-      e_grow = grow;
-      e_h = h;
+      const uint32_t last = sc0 + L - 1, is = it & 1;
+      if ((last & 1) != wgi) {
+        // the other warpgroup finishes the item: hand it this one's normaliser
+        *const_cast<volatile float*>(&sm.l_row[is][row]) = l;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.l_full[is][quarter]);
+      } else {
+        // epilogue: O / l -> bf16, LSE (natural log)
+        if (!(ok = warp_wait(&sm.l_full[is][quarter], (it >> 1) & 1, abort_flag, prm.status, prm.timeout_ns))) break;
+        const float l_o = *const_cast<volatile float*>(&sm.l_row[is][row]);
+        // it is under the maximum that the last tile but one used, <= m
+        if (l_o > 0.f) l += l_o * ex2_approx(m_before - m);
+        if (!(ok = warp_wait(&sm.pv_done[last & 1], (last >> 1) & 1, abort_flag, prm.status, prm.timeout_ns))) break;
+        tc_fence_after();
+        uint32_t o[D];
+#pragma unroll
+        for (int g = 0; g < D / 32; ++g)
+          tmem_ld32(tmem + lane_base + kColO + g * 32, *reinterpret_cast<uint32_t(*)[32]>(&o[g * 32]));
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.o_empty);
+        const float inv = (!kSub || l > 0.f) ? 1.0f / l : 0.f;  // a row that saw no key: O = 0, LSE = -inf
+        if (row_ok) {
+#pragma unroll
+          for (int x = 0; x < D; x += 8) {
+            uint4 v;
+            v.x = pack_bf16x2(__uint_as_float(o[x + 0]) * inv, __uint_as_float(o[x + 1]) * inv);
+            v.y = pack_bf16x2(__uint_as_float(o[x + 2]) * inv, __uint_as_float(o[x + 3]) * inv);
+            v.z = pack_bf16x2(__uint_as_float(o[x + 4]) * inv, __uint_as_float(o[x + 5]) * inv);
+            v.w = pack_bf16x2(__uint_as_float(o[x + 6]) * inv, __uint_as_float(o[x + 7]) * inv);
+            *reinterpret_cast<uint4*>(orow + x) = v;
+          }
+          prm.lse[(int64_t)h * prm.N + grow] = (!kSub || l > 0.f) ? (m + log2f(l)) * 0.69314718055994531f : -INFINITY;
+        }
+      }
       sc0 += L;
+      ++it;
     }
-    if (ok && pend) ok = epilogue();
   }
 
   tc_fence_before();
@@ -494,16 +595,22 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
   if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
-static_assert(sizeof(FwdSmem<128>) + 1024 <= 232448, "forward shared layout exceeds the per-block limit");
+static_assert(sizeof(FwdSmem<128>) <= 232448, "forward shared layout exceeds the per-block limit");
 
 template <int D, int kMode>
 static cudaError_t launch_d(const AttnProblem& p, const CUtensorMap& tq, const CUtensorMap& tk,
                             const CUtensorMap& tv, const CUtensorMap& tk64, const CUtensorMap& tv64,
                             const FwdParams& prm, int grid, cudaStream_t stream) {
-  const size_t smem = sizeof(FwdSmem<D>) + 1024;
+  const size_t smem = sizeof(FwdSmem<D>);
   cudaError_t e =
       cudaFuncSetAttribute(attn_fwd_tc_kernel<D, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  // the setmaxnreg split assumes exactly kFwdRegLaunch registers per thread at
+  // launch: with fewer, the increases would wait for registers that never come
+  cudaFuncAttributes fa;
+  e = cudaFuncGetAttributes(&fa, attn_fwd_tc_kernel<D, kMode>);
+  if (e != cudaSuccess) return e;
+  if (fa.numRegs != kFwdRegLaunch) return cudaErrorInvalidConfiguration;
   attn_fwd_tc_kernel<D, kMode><<<grid, kFwdThreads, smem, stream>>>(tq, tk, tv, tk64, tv64, prm);
   return cudaGetLastError();
 }

@@ -1,6 +1,7 @@
-"""GPU parity of the attention kernels' schedules: lists of very unequal length
-(the backward's longest-first order) and a backward workspace without room for
-that order."""
+"""GPU parity of the attention kernels' schedules: many items per CTA with lists
+of 0, 1, 2 and more blocks (the forward's stream of key tiles crosses item
+boundaries with every parity), lists of very unequal length (the backward's
+longest-first order) and a backward workspace without room for that order."""
 import ctypes
 
 import numpy as np
@@ -33,6 +34,38 @@ def _problem(N, H, d, bq, bk, lengths, seed):
             n = min(nk, lengths[(h * nq + i) % len(lengths)])
             bm[h, i, g.choice(nk, size=n, replace=False)] = 1
     return x, bm
+
+
+def _reference(x, bm, bq, bk):
+    """O and LSE by the definition, every score in 64 bits."""
+    q, k, v = (t.double() for t in x[:3])
+    N, H, d = q.shape
+    keep = torch.from_numpy(np.repeat(np.repeat(bm, bq, 1), bk, 2)[:, :N, :N]).cuda().bool()
+    s = torch.einsum("nhd,mhd->hnm", q, k) * d ** -0.5
+    s = s.masked_fill(~keep, -float("inf"))
+    lse = torch.logsumexp(s, 2)
+    p = torch.nan_to_num(torch.exp(s - lse[:, :, None]))
+    return torch.einsum("hnm,mhd->nhd", p, v), lse
+
+
+LENGTHS = [(1,), (2,), (1, 2, 3), (0, 1, 0, 2, 5), (4, 1, 1, 7)]
+
+
+@pytest.mark.parametrize("lengths", LENGTHS, ids=lambda x: "-".join(map(str, x)))
+@pytest.mark.parametrize("d,bq,bk", [(128, 128, 128), (64, 128, 128), (128, 64, 64), (128, 128, 64), (64, 64, 128)])
+def test_forward_short_lists_many_items(d, bq, bk, lengths):
+    from paper_2609_23169_gb300 import ultratex as u
+    N, H = 1000, 40  # 320 items of 128 rows: two or three per CTA, the last block ragged
+    x, bm = _problem(N, H, d, bq, bk, lengths, 1)
+    st = u.status_word()
+    o, lse = u.ut_bsattn_fwd(*x[:3], *_lists(bm), bq, status=st, block_k=bk)
+    ref_o, ref_l = _reference(x, bm, bq, bk)
+    assert int(st.item()) == 0
+    assert_bf16_close(to_np(o), ref_o.cpu().numpy(), "O")
+    got, want = to_np(lse), ref_l.cpu().numpy()
+    assert np.array_equal(np.isfinite(got), np.isfinite(want))
+    fin = np.isfinite(want)
+    assert np.abs(got[fin] - want[fin]).max(initial=0.0) <= 1e-4
 
 
 @pytest.mark.parametrize("d,bq,bk", [(128, 128, 128), (64, 64, 64)])
