@@ -59,7 +59,7 @@ struct AttnProblem {
   int nk;        // key blocks (rows of the transposed lists per head)
 };
 
-// attn_simt.cu (fp32 path and the generic CUDA-core backward)
+// attn_simt.cu (fp32 path)
 cudaError_t launch_attn_fwd_simt(const AttnProblem& p, const void* q, const void* k, const void* v,
                                  const int32_t* row_ptr, const int32_t* col_idx, void* o, float* lse,
                                  cudaStream_t stream);

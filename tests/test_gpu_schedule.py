@@ -102,3 +102,54 @@ def test_backward_order_and_workspace(d, bq, bk):
     torch.einsum("hnm,mhd->nhd", p, v).backward(x[3].double())
     for got, ref, name in zip(out[0], (q.grad, k.grad, v.grad), ("dQ", "dK", "dV")):
         assert_bf16_close(to_np(got), ref.cpu().numpy(), name)
+
+
+@pytest.mark.parametrize("N,H,d,b", [(1, 1, 64, 32), (33, 2, 128, 32), (130, 1, 64, 128), (200, 3, 128, 64),
+                                     (611, 2, 64, 32), (611, 1, 128, 128)])
+@pytest.mark.parametrize("aligned", [True, False])
+def test_fp32_pieces_and_alignment(N, H, d, b, aligned):
+    """fp32 forward and backward at the edges of the 32-row pieces (blocks whose
+    last pieces do not exist, lists of odd piece counts, empty lists) and, in
+    the backward, tensors aligned to 4 bytes only."""
+    from paper_2609_23169_gb300 import ultratex as u
+    g = np.random.Generator(np.random.PCG64([79, N]))
+    x = [torch.from_numpy(g.standard_normal((N, H, d)).astype(np.float32)).cuda() for _ in range(4)]
+    nb = -(-N // b)
+    bm = (g.random((H, nb, nb)) < 0.6).astype(np.uint8)
+    bm[0, 0] = 0
+    if nb > 1:
+        bm[0, 1, nb - 1] = 1
+    csr, csc = _lists(bm), _lists(np.ascontiguousarray(bm.transpose(0, 2, 1)))
+    if csr[1].numel() == 0:
+        csr, csc = (csr[0], torch.zeros(1, dtype=torch.int32, device="cuda")), (csc[0], torch.zeros(1, dtype=torch.int32, device="cuda"))
+    st = u.status_word()
+    o, lse = u.ut_bsattn_fwd(*x[:3], *csr, b, status=st)
+
+    def place(t):
+        if aligned:
+            return t
+        flat = torch.empty(t.numel() + 4, dtype=t.dtype, device="cuda")[1:1 + t.numel()].view(t.shape)
+        flat.copy_(t)
+        return flat
+
+    grads = [place(torch.zeros_like(x[0])) for _ in range(3)]
+    y = [place(t) for t in x]
+    u.ut_bsattn_bwd(y[0], y[1], y[2], place(o), lse, y[3], *csr, *csc, b, dq=grads[0], dk=grads[1], dv=grads[2], status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    q, k, v = (t.double().requires_grad_(True) for t in x[:3])
+    keep = torch.from_numpy(np.repeat(np.repeat(bm, b, 1), b, 2)[:, :N, :N]).cuda().bool()
+    s = (torch.einsum("nhd,mhd->hnm", q, k) * d ** -0.5).masked_fill(~keep, -float("inf"))
+    seen = keep.any(2)[:, :, None]
+    p = torch.softmax(s.masked_fill(~seen, 0.0), 2) * seen
+    ref = torch.einsum("hnm,mhd->nhd", p, v)
+    ref.backward(x[3].double())
+    # 1e-5 is the stated fp32 tolerance; the sums here have at most 611 terms of order one
+    assert np.abs(to_np(o) - ref.detach().cpu().numpy()).max() <= 1e-5
+    want = torch.logsumexp(s, 2).detach().cpu().numpy()
+    got = to_np(lse)
+    assert np.array_equal(np.isneginf(got), np.isneginf(want))
+    fin = np.isfinite(want)
+    assert np.abs(got[fin] - want[fin]).max(initial=0.0) <= 1e-5
+    for gg, rr, name in zip(grads, (q.grad, k.grad, v.grad), ("dQ", "dK", "dV")):
+        assert np.abs(to_np(gg) - rr.cpu().numpy()).max() <= 2e-5, name
