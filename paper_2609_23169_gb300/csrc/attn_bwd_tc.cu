@@ -106,7 +106,7 @@ UT_DEV void order_group(const OrderParams& o, int g) {
   for (int x = threadIdx.x; x < n; x += blockDim.x) o.order[first + atomicAdd(&bins[bin(x)], 1)] = first + x;
 }
 
-// D_r = dO_r . O_r and LSE_r * log2(e) into the padded [H, Np] workspace, and the
+// -D_r = -dO_r . O_r and -LSE_r * log2(e) into the padded [H, Np] workspace, and the
 // dQ accumulator's row cleared; one warp per row r of Np.  The first
 // o.groups blocks write the item order instead.
 __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __restrict__ o,
@@ -149,8 +149,8 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
     }
     for (int off = lanes_per_head / 2; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if ((lane % lanes_per_head) == 0 && h < H) {
-      dsum[(int64_t)h * Np + r] = r < N ? s : 0.f;
-      lse2[(int64_t)h * Np + r] = r < N ? lse[(int64_t)h * N + r] * 1.4426950408889634f : INFINITY;
+      dsum[(int64_t)h * Np + r] = r < N ? -s : 0.f;
+      lse2[(int64_t)h * Np + r] = r < N ? lse[(int64_t)h * N + r] * -1.4426950408889634f : -INFINITY;
     }
   }
 }
@@ -158,8 +158,8 @@ __global__ void __launch_bounds__(256) bwd_pre_kernel(const __nv_bfloat16* __res
 struct BwdParams {
   const int32_t* ptr;   // transposed fine lists: per (head, key block) the query blocks
   const int32_t* idx;
-  const float* lse2;    // [H, Np]  LSE * log2(e)
-  const float* dsum;    // [H, Np]  D
+  const float* lse2;    // [H, Np]  -LSE * log2(e) (padding rows: -inf, so that P = 0)
+  const float* dsum;    // [H, Np]  -D
   __nv_bfloat16* out0;  // dv
   __nv_bfloat16* out1;  // dk
   int32_t* status;
@@ -219,9 +219,9 @@ constexpr uint32_t kColR0 = 0, kColRQ = 128, kColFuDv = 256, kColFuDk = 384;
 // 36-153 query blocks per key block at the 2048 canvas, so a static
 // round-robin leaves the busiest CTA ~5% above the mean), still in head-major
 // order, so that the CTAs in flight share one head's Q, dO and dQ accumulator
-// in L2.  kItemConsumers: TMA lane 1, the MMA warp, 8 elementwise warps, 4
+// in L2.  kItemConsumers: TMA lane 1, the row-vector producer, the MMA warp, 8 elementwise warps, 4
 // drain warps.
-constexpr int kItemSlots = 4, kItemConsumers = 14;
+constexpr int kItemSlots = 4, kItemConsumers = 15;
 
 template <int D>
 struct FusedSmem {
@@ -233,13 +233,13 @@ struct FusedSmem {
   alignas(1024) uint8_t dst[kTile * kTile * 2];  // dS^T of the current pair
   alignas(1024) uint8_t q[kFuQStages][kTileBytes];
   alignas(1024) uint8_t dout[kFuDoStages][kTileBytes];
-  alignas(16) float lse2[2][kTile];
+  alignas(16) float lse2[2][kTile];           // -LSE log2 e and -D of the pair's query rows
   alignas(16) float dsum[2][kTile];
   uint64_t kv_full, kv_empty;
   uint64_t q_full[kFuQStages], q_empty[kFuQStages], do_full[kFuDoStages], do_empty[kFuDoStages];
   uint64_t s_full, s_empty, dp_full, dp_empty, pt_full, pt_done, dst_full, ds_done, dq_empty;
   uint64_t acc_full, acc_empty, mma_done;
-  uint64_t rowvec_full[2];
+  uint64_t vec_full[2], vec_empty[2];
   // the CTA's item sequence: TMA lane 0 takes the next item from the global
   // counter and publishes it here; every other role reads the slots in order
   int32_t item[kItemSlots];
@@ -297,8 +297,10 @@ __global__ void __launch_bounds__(kFuThreads, 1)
     mbar_init(&sm.acc_full, 1);
     mbar_init(&sm.acc_empty, 8);
     mbar_init(&sm.mma_done, 1);
-    mbar_init(&sm.rowvec_full[0], 256);
-    mbar_init(&sm.rowvec_full[1], 256);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&sm.vec_full[s], 1);
+      mbar_init(&sm.vec_empty[s], 8);
+    }
     for (int s = 0; s < kItemSlots; ++s) {
       mbar_init(&sm.item_full[s], 1);
       mbar_init(&sm.item_empty[s], kItemConsumers);
@@ -411,6 +413,37 @@ __global__ void __launch_bounds__(kFuThreads, 1)
         if (ki > 0) drain(&sm.kv_full, (ki - 1) & 1);
         for (uint32_t u = (qd >= nst ? qd - nst : 0); u < qd; ++u) drain(&full[u % nst], (u / nst) & 1);
       }
+    } else if (warp == 2) {
+      // row vectors of the pair's query rows, two pairs ahead (freed by the
+      // elementwise warps): fetched by those warps themselves and handed round
+      // through shared memory they cost ~480 of ~5,100 cycles of every pair
+      // (2048 canvas, backward: 22.23 -> 21.6 ms)
+      if (lane == 0) {
+        uint32_t qd = 0, kk = 0;
+        bool ok = true;
+        while (ok) {
+          int w;
+          if (!(ok = next_item(kk, w, true)) || w < 0) break;
+          const int64_t base = (int64_t)(w / prm.nq) * prm.Np;
+          BlockSteps<kMode> tl;
+          tl.init(prm.ptr, prm.idx, w / prm.nq, w % prm.nq, prm.nk_fine, prm.k_rows_per_tile, prm.list_shift);
+          int i, ih;
+          uint32_t bits;
+          for (; tl.next(i, ih, bits); ++qd) {
+            const uint32_t st = qd & 1;
+            if (!(ok = mbar_wait(&sm.vec_empty[st], ((qd >> 1) & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns))) break;
+            const int64_t b0 = base + 64 * (int64_t)(tl.pair ? PairList::load_lo(i, ih) : 2 * i);
+            const int64_t b1 = base + 64 * (int64_t)(tl.pair ? PairList::load_hi(i, ih) : 2 * i + 1);
+            mbar_expect_tx(&sm.vec_full[st], 2 * kTile * sizeof(float));
+            bulk_load(&sm.lse2[st][0], prm.lse2 + b0, 256, &sm.vec_full[st]);
+            bulk_load(&sm.lse2[st][64], prm.lse2 + b1, 256, &sm.vec_full[st]);
+            bulk_load(&sm.dsum[st][0], prm.dsum + b0, 256, &sm.vec_full[st]);
+            bulk_load(&sm.dsum[st][64], prm.dsum + b1, 256, &sm.vec_full[st]);
+          }
+        }
+        for (uint32_t u = (qd >= 2 ? qd - 2 : 0); u < qd; ++u)
+          if (!mbar_drain(&sm.vec_full[u & 1], (u >> 1) & 1, kDrainTimeoutNs)) set_status(prm.status, UT_ERR_TIMEOUT);
+      }
     } else if (warp == 1) {
       // whole warp, converged: waits are warp-uniform, MMAs/commits elect one lane.
       // Per pair t: dP^T_t, dV_t, S^T_{t+1}, dK_t, dQ_t^T.
@@ -513,7 +546,6 @@ __global__ void __launch_bounds__(kFuThreads, 1)
     const uint32_t quarter = warp & 3;
     const uint32_t half = (warp - 4) >> 2;
     const uint32_t krow = quarter * 32 + lane;  // key row of the tile = TMEM lane (d index for dQ^T)
-    const uint32_t tid = threadIdx.x - 128;     // 0..255 within the elementwise group
     const uint32_t lane_base = (quarter * 32) << 16;
     constexpr int HC = kTile / 2;               // query columns per half
     constexpr int HD = D / 2;                   // output columns per half
@@ -542,33 +574,18 @@ __global__ void __launch_bounds__(kFuThreads, 1)
           }
         continue;
       }
-      // this thread's element of the query-row vectors (LSE*log2e for threads
-      // 0-127, D for 128-255) is loaded one pair ahead: query column
-      // tid mod 128 of the tile, in its 64-row half
-      const uint32_t qcol = tid & (kTile - 1), qhalf = qcol >> 6;
-      const float* rv_src = (tid < kTile ? prm.lse2 : prm.dsum) + (int64_t)h * prm.Np + (qcol & 63);
-      auto rv_row = [&](int lo, int hi) -> int64_t {  // first row of this thread's 64-row query half
-        if (tl.pair) return 64 * (int64_t)(qhalf ? PairList::load_hi(lo, hi) : PairList::load_lo(lo, hi));
-        return (int64_t)lo * kTile + 64 * qhalf;
-      };
-      int i_next, ih_next;
-      uint32_t bits_next;
-      tl.next(i_next, ih_next, bits_next);
-      float rv = rv_src[rv_row(i_next, ih_next)];
       for (int t = 0; t < L; ++t) {
         const uint32_t qd = qd0 + t;
         // this half's 64 query columns and this thread's 64 key rows form one
         // 64 x 64 sub-block of the tile pair: listed or not
-        const bool listed = !kSub || ((bits_next >> (2 * kh + half)) & 1u);
-        // this pair's query-row LSE*log2e and D into the shared double buffer
-        // (buffer qd&1 was last read in pair qd-2, which every thread finished
-        //  before arriving for pair qd-1)
-        if (tid < kTile) sm.lse2[qd & 1][tid] = rv;
-        else sm.dsum[qd & 1][tid - kTile] = rv;
-        mbar_arrive(&sm.rowvec_full[qd & 1]);
-        if (t + 1 < L && tl.next(i_next, ih_next, bits_next)) rv = rv_src[rv_row(i_next, ih_next)];
-        if (!(ok = warp_wait(&sm.rowvec_full[qd & 1], (qd >> 1) & 1, abort_flag, prm.status, prm.timeout_ns)))
-          break;
+        bool listed = true;
+        if (kSub) {
+          int i, ih;
+          uint32_t bits;
+          tl.next(i, ih, bits);
+          listed = (bits >> (2 * kh + half)) & 1u;
+        }
+        if (!(ok = warp_wait(&sm.vec_full[qd & 1], (qd >> 1) & 1, abort_flag, prm.status, prm.timeout_ns))) break;
         const float* ls = sm.lse2[qd & 1] + half * HC;
         const float* ds_v = sm.dsum[qd & 1] + half * HC;
         if (!(ok = warp_wait(&sm.s_full, qd & 1, abort_flag, prm.status, prm.timeout_ns))) break;
@@ -584,10 +601,14 @@ __global__ void __launch_bounds__(kFuThreads, 1)
 #pragma unroll
             for (int x = 0; x < HC; x += 4) {
               const float4 l4 = *reinterpret_cast<const float4*>(ls + x);
-              p[x + 0] = ex2_approx(fmaf(__uint_as_float(r[x + 0]), c, -l4.x));
-              p[x + 1] = ex2_approx(fmaf(__uint_as_float(r[x + 1]), c, -l4.y));
-              p[x + 2] = ex2_approx(fmaf(__uint_as_float(r[x + 2]), c, -l4.z));
-              p[x + 3] = ex2_approx(fmaf(__uint_as_float(r[x + 3]), c, -l4.w));
+              const float2 e0 = ffma2(make_float2(__uint_as_float(r[x]), __uint_as_float(r[x + 1])), make_float2(c, c),
+                                      make_float2(l4.x, l4.y));
+              const float2 e1 = ffma2(make_float2(__uint_as_float(r[x + 2]), __uint_as_float(r[x + 3])),
+                                      make_float2(c, c), make_float2(l4.z, l4.w));
+              p[x + 0] = ex2_approx(e0.x);
+              p[x + 1] = ex2_approx(e0.y);
+              p[x + 2] = ex2_approx(e1.x);
+              p[x + 3] = ex2_approx(e1.y);
             }
           } else {
 #pragma unroll
@@ -623,9 +644,14 @@ __global__ void __launch_bounds__(kFuThreads, 1)
           for (int x = 0; x < 32; x += 4) {
             const float4 d4 = *reinterpret_cast<const float4*>(ds_v + hh * 32 + x);
             const float* pp = p + hh * 32 + x;
-            dsk[x / 2] = pack_bf16x2(pp[0] * (__uint_as_float(r[x]) - d4.x), pp[1] * (__uint_as_float(r[x + 1]) - d4.y));
-            dsk[x / 2 + 1] =
-                pack_bf16x2(pp[2] * (__uint_as_float(r[x + 2]) - d4.z), pp[3] * (__uint_as_float(r[x + 3]) - d4.w));
+            const float2 a0 = mul2(make_float2(pp[0], pp[1]),
+                                   add2(make_float2(__uint_as_float(r[x]), __uint_as_float(r[x + 1])),
+                                        make_float2(d4.x, d4.y)));
+            const float2 a1 = mul2(make_float2(pp[2], pp[3]),
+                                   add2(make_float2(__uint_as_float(r[x + 2]), __uint_as_float(r[x + 3])),
+                                        make_float2(d4.z, d4.w)));
+            dsk[x / 2] = pack_bf16x2(a0.x, a0.y);
+            dsk[x / 2 + 1] = pack_bf16x2(a1.x, a1.y);
           }
           if (hh == 0 && !(ok = warp_wait(&sm.ds_done, (qd & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns)))
             break;
@@ -639,7 +665,10 @@ __global__ void __launch_bounds__(kFuThreads, 1)
         if (!ok) break;
         fence_proxy_async_smem();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.dst_full);
+        if (lane == 0) {
+          mbar_arrive(&sm.dst_full);
+          mbar_arrive(&sm.vec_empty[qd & 1]);
+        }
       }
       if (!ok) break;
       if (!(ok = warp_wait(&sm.acc_full, ki & 1, abort_flag, prm.status, prm.timeout_ns))) break;
