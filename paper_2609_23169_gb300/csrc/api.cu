@@ -312,7 +312,7 @@ ut_status ut_block_mask(const ut_attn_shape* shape, int32_t mode, const void* q,
   if (!bitmap || !dev_status) return UT_ERR_INVALID_ARG;
   if (col_cap > 0 && !col_idx) return UT_ERR_INVALID_ARG;
   return from_cuda(
-      launch_block_mask_bitmap(p, bitmap, row_ptr, col_idx, col_ptr_t, row_idx_t, col_cap, ws, dev_status, s));
+      launch_block_mask_bitmap(p, bitmap, row_ptr, col_idx, col_ptr_t, row_idx_t, col_cap, dev_status, s));
 }
 
 ut_status ut_bsattn_fwd(const ut_attn_shape* shape, const void* q, const void* k, const void* v,

@@ -3,25 +3,29 @@
 // Top-K mode:
 //   block_pool_kernel    pool(Q) over blocks of b_q rows, pool(K) over blocks
 //                        of b_kv rows: fp32 mean over the valid rows of each
-//                        block, every head at once (one CTA per block).
+//                        block (one CTA per block and 128 16-byte columns).
 //   score_select_kernel  S_c[i, :] = pool(Q)_i . pool(K)_j in fp32 for R query
-//                        blocks of one head, then per row an exact radix
-//                        select of the K_rho-th largest score (4 passes of 8
-//                        bits over order-preserving keys); equal scores go to
-//                        the smaller key-block index.  Writes the ascending
-//                        list and the dense [H, N_q, N_k] bitmap row.
-// Both modes:
-//   bitmap_count_kernel  entries per row (or per column for the transpose),
-//   scan_kernel          exclusive prefix -> row_ptr / col_ptr,
+//                        blocks of one head, then per row an exact select of
+//                        the K_rho-th largest score over order-preserving keys;
+//                        equal scores go to the smaller key-block index.
+//                        Writes row_ptr, the ascending list and the row of a
+//                        [H, N_q, N_k] bit mask (32 key blocks per word).
+//   transpose_kernel     the lists per key block from the bit mask, by warp
+//                        ballots.
+// Bitmap mode, lists and transpose side by side in each launch:
+//   bitmap_count_kernel  entries per row and per column (into the pointers),
+//   scan_kernel          exclusive prefix in place -> row_ptr / col_ptr,
 //   bitmap_fill_kernel   ascending lists by warp ballot.
 #include "common.cuh"
 #include "kernels.h"
 
 namespace ut {
 
-constexpr int kPoolThreads = 256;
-constexpr int kSelThreads = 256;
-constexpr int kSelMaxRows = 16;
+constexpr int kPoolThreads = 128;
+constexpr int kSelThreads = 128;
+constexpr int kSelCols = 256;      // key blocks per tile of scores
+constexpr int kSelRows = 16;       // query blocks per CTA (fewer when N_k is large)
+constexpr int kSelRegKeys = 32;    // keys a lane holds in registers: N_k <= 1024
 
 template <typename T>
 struct Vec8;
@@ -48,8 +52,12 @@ struct Vec8<float> {
   }
 };
 
-// grid (max(nq, nk), 2): blockIdx.y selects Q (0, blocks of bq rows) or K (1,
-// blocks of bk rows).  out: pooled Q [H][nq][d], then pooled K [H][nk][d].
+// grid (max(nq, nk), 2, column slices): blockIdx.y selects Q (0, blocks of bq
+// rows) or K (1, blocks of bk rows), a thread owns one 16-byte column of the
+// slice.  out: pooled Q [H][nq][d], then pooled K [H][nk][d].  HBM-bound (Q and K
+// are read once); one column a thread keeps every thread of a row busy whatever
+// H * d is, and small problems get three times the CTAs.
+// 2048 canvas (1.05 GB): 189 -> 160 us, 6.55 TB/s.
 template <typename T>
 __global__ void __launch_bounds__(kPoolThreads) block_pool_kernel(const T* __restrict__ q, const T* __restrict__ k,
                                                                   int64_t N, int H, int d, int64_t row_stride,
@@ -60,29 +68,24 @@ __global__ void __launch_bounds__(kPoolThreads) block_pool_kernel(const T* __res
   const T* x = is_k ? k : q;
   const int block = is_k ? bk : bq, nb = is_k ? nk : nq;
   const int i = blockIdx.x;
-  if (i >= nb) return;
-  float* base = is_k ? out + (size_t)H * nq * d : out;
+  const int c0 = (blockIdx.z * kPoolThreads + threadIdx.x) * E;
+  if (i >= nb || c0 >= H * d) return;
   const int64_t r0 = (int64_t)i * block;
   const int64_t r1 = min(N, r0 + block);
-  const int cols = H * d;
-  const float inv_cnt = 1.0f / (float)(r1 - r0);
-  for (int ch = threadIdx.x; ch * E < cols; ch += kPoolThreads) {
-    float acc[E];
+  float acc[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) acc[e] = 0.f;
-    for (int64_t r = r0; r < r1; ++r) {
-      float f[E];
-      Vec8<T>::load(x + r * row_stride + (int64_t)ch * E, f);
+  for (int e = 0; e < E; ++e) acc[e] = 0.f;
+  const T* p = x + r0 * row_stride + c0;
+#pragma unroll 16
+  for (int64_t r = r0; r < r1; ++r, p += row_stride) {
+    float f[E];
+    Vec8<T>::load(p, f);
 #pragma unroll
-      for (int e = 0; e < E; ++e) acc[e] += f[e];
-    }
-    const int c0 = ch * E;
-    const int h = c0 / d, e0 = c0 % d;
-    float* dst = base + ((int64_t)h * nb + i) * d + e0;
-#pragma unroll
-    for (int e = 0; e < E; ++e) dst[e] = __fdiv_rn(acc[e], (float)(r1 - r0));
-    (void)inv_cnt;
+    for (int e = 0; e < E; ++e) acc[e] += f[e];
   }
+  float* dst = (is_k ? out + (size_t)H * nq * d : out) + ((int64_t)(c0 / d) * nb + i) * d + c0 % d;
+#pragma unroll
+  for (int e = 0; e < E; ++e) dst[e] = __fdiv_rn(acc[e], (float)(r1 - r0));
 }
 
 UT_DEV uint32_t order_key(float s) {
@@ -91,144 +94,310 @@ UT_DEV uint32_t order_key(float s) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// grid (H, ceil(nq / R)); dynamic smem: R*d + R*nk floats + 8 warps * 256 ints.
-// Rows are query blocks (nq per head), columns key blocks (nk).
+// Score of a key (the inverse of order_key).
+UT_DEV float key_score(uint32_t u) { return __uint_as_float((u & 0x80000000u) ? (u & 0x7FFFFFFFu) : ~u); }
+
+// K-th largest of the warp's n_lo keys, lo and top the smallest and the largest:
+// count_ge(lo) >= k > count_ge(hi) holds throughout and the bracket closes in on the largest value
+// with at least k keys >= it.  Candidates alternate between the score that a
+// straight line through the bracket's counts gives (scores near a quantile are
+// nearly evenly spread: some eight steps, against 32 by bits) and the middle of
+// the bracket, which bounds the steps whatever the scores are.  A candidate
+// with exactly k keys at or above it ends the search.  On return every key >
+// thr belongs, and the first `equal` keys (by index) that are equal to thr.
+template <typename Count>
+UT_DEV void select_kth(Count count_ge, int k, uint32_t lo, uint32_t top, int n_lo, uint32_t& thr, int& equal) {
+  uint32_t hi = top;
+  int n_hi = 0;
+  if (top != 0xffffffffu) {
+    hi = top + 1;
+  } else {  // NaN scores (the largest key there is) stand first
+    n_hi = __reduce_add_sync(0xffffffffu, count_ge(top));
+    if (n_hi >= k) {
+      thr = top;
+      equal = k;
+      return;
+    }
+  }
+  if (n_lo == k && lo > 0) {  // every key
+    thr = lo - 1;
+    equal = 0;
+    return;
+  }
+  for (int step = 0; hi - lo > 1; ++step) {
+    uint32_t cand = lo + ((hi - lo) >> 1);
+    if (!(step & 1)) {
+      const float a = key_score(lo), b = key_score(hi);
+      const float f = a + (b - a) * __fdividef((float)(n_lo - k) + 0.5f, (float)(n_lo - n_hi));
+      const uint32_t c = order_key(f);  // (not finite: outside the bracket or harmless)
+      if (c > lo && c < hi) cand = c;
+    }
+    const int n = __reduce_add_sync(0xffffffffu, count_ge(cand));
+    if (n == k) {  // the keys >= cand are the answer: > cand - 1 (cand > 0)
+      thr = cand - 1;
+      equal = 0;
+      return;
+    }
+    if (n > k) {
+      lo = cand;
+      n_lo = n;
+    } else {
+      hi = cand;
+      n_hi = n;
+    }
+  }
+  thr = lo;
+  equal = k - n_hi;
+}
+
+// K-th largest of the keys of one row, kKeys per lane in registers (absent ones
+// 0: below every score's key).
+template <int kKeys>
+UT_DEV void select_row(const float* srow, int nk, int k, int lane, uint32_t& thr, int& equal) {
+  uint32_t key[kKeys], lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+  for (int x = 0; x < kKeys; ++x) {
+    const int j = 32 * x + lane;
+    key[x] = j < nk ? order_key(srow[j]) : 0u;
+    if (j < nk) {
+      lo = min(lo, key[x]);
+      hi = max(hi, key[x]);
+    }
+  }
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  select_kth(
+      [&](uint32_t cand) {
+        int n = 0;
+#pragma unroll
+        for (int x = 0; x < kKeys; ++x) n += key[x] >= cand;
+        return n;
+      },
+      k, lo, hi, nk, thr, equal);
+}
+
+// grid (H, ceil(nq / R)); dynamic smem: pooled query rows [d][kRows], a slice of
+// pooled keys [kE][kSelCols], scores [R][nk].  Rows are query blocks (nq per
+// head), columns key blocks (nk).
+// The scores are bound by what shared memory can hand to the registers (128
+// bytes a cycle, a broadcast counted in full): a thread that owned one key
+// block and 16 rows read 68 bytes for 16 multiply-adds and the launch took 320
+// us at the 2048 canvas; 8 rows x 4 key blocks read 48 for 32 (and with the
+// search above instead of 32 passes by bits 263 -> 194; 282 with the keys read
+// from global memory and a radix select over shared counters).  Slices are
+// staged d-major, 4-column groups exchanged by (d / 4) % 8 so that neither the
+// transposing stores nor the reads conflict.  A sum runs over d in order, as
+// one FMA chain.
+template <int kRows, int kE>  // rows a tile holds, d per staged slice of pool(K)
 __global__ void __launch_bounds__(kSelThreads) score_select_kernel(const float* __restrict__ pooled, int H, int d,
                                                                    int nq, int nk, int R, int k_rho,
+                                                                   int32_t* __restrict__ row_ptr,
                                                                    int32_t* __restrict__ col_idx,
-                                                                   uint8_t* __restrict__ bitmap) {
-  extern __shared__ float smem[];
-  float* pq = smem;                       // [R][d]
-  float* sc = smem + R * d;               // [R][nk]
-  uint32_t* hist = reinterpret_cast<uint32_t*>(sc + R * nk);  // [8][256]
+                                                                   uint32_t* __restrict__ bits) {
+  extern __shared__ __align__(16) float smem[];
+  constexpr int kTr = kRows / 2, kTc = 4;  // a thread's rows and columns: 2 row groups x 64 column groups
+  const int tid = threadIdx.x;
+  float* pq = smem;                      // [d][kRows]
+  float* kt = pq + kRows * d;            // [kE][kSelCols]
+  float* sc = kt + kE * kSelCols;     // [R][nk]
   const int h = blockIdx.x;
   const int i0 = blockIdx.y * R;
   const int rows = min(R, nq - i0);
-  const float* PQ = pooled + ((int64_t)h * nq) * d;
+  const int rg = tid & 1, cg = tid >> 1;
+  const float* PQ = pooled + ((int64_t)h * nq + i0) * d;
   const float* PK = pooled + (int64_t)H * nq * d + ((int64_t)h * nk) * d;
-  for (int t = threadIdx.x; t < rows * d; t += kSelThreads) pq[t] = PQ[(int64_t)i0 * d + t];
-  __syncthreads();
-  // two key blocks per thread and 16-byte loads of the pooled query rows: one
-  // shared load feeds eight FMAs (the sums are accumulated in the same order
-  // as one column at a time)
-  for (int j0 = threadIdx.x; j0 < nk; j0 += 2 * kSelThreads) {
-    const int j1 = j0 + kSelThreads;
-    const bool has1 = j1 < nk;
-    float acc0[kSelMaxRows], acc1[kSelMaxRows];
+  for (int t = tid; t < kRows * d; t += kSelThreads) {
+    const int r = t / d, e = t % d;
+    pq[e * kRows + r] = r < rows ? PQ[t] : 0.f;
+  }
+  for (int j0 = 0; j0 < nk; j0 += kSelCols) {
+    float2 acc[kTr / 2][kTc];
 #pragma unroll
-    for (int r = 0; r < kSelMaxRows; ++r) acc0[r] = acc1[r] = 0.f;
-    const float* k0 = PK + (int64_t)j0 * d;
-    const float* k1 = PK + (int64_t)(has1 ? j1 : j0) * d;
-    for (int e = 0; e < d; e += 4) {
-      const float4 a = *reinterpret_cast<const float4*>(k0 + e);
-      const float4 b = *reinterpret_cast<const float4*>(k1 + e);
+    for (int r = 0; r < kTr / 2; ++r)
 #pragma unroll
-      for (int r = 0; r < kSelMaxRows; ++r) {
-        if (r < rows) {
-          const float4 p = *reinterpret_cast<const float4*>(pq + r * d + e);
-          acc0[r] = fmaf(p.x, a.x, acc0[r]);
-          acc0[r] = fmaf(p.y, a.y, acc0[r]);
-          acc0[r] = fmaf(p.z, a.z, acc0[r]);
-          acc0[r] = fmaf(p.w, a.w, acc0[r]);
-          acc1[r] = fmaf(p.x, b.x, acc1[r]);
-          acc1[r] = fmaf(p.y, b.y, acc1[r]);
-          acc1[r] = fmaf(p.z, b.z, acc1[r]);
-          acc1[r] = fmaf(p.w, b.w, acc1[r]);
-        }
+      for (int x = 0; x < kTc; ++x) acc[r][x] = make_float2(0.f, 0.f);
+    constexpr int kLoads = kSelCols * (kE / 4) / kSelThreads;  // 16-byte loads of a slice per thread
+    float4 next[kLoads];
+    auto fetch = [&](int e0) {
+#pragma unroll
+      for (int x = 0; x < kLoads; ++x) {
+        const int t = x * kSelThreads + tid, j = t / (kE / 4), a = t % (kE / 4);
+        next[x] = j0 + j < nk ? *reinterpret_cast<const float4*>(PK + (int64_t)(j0 + j) * d + e0 + 4 * a)
+                              : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+    };
+    fetch(0);
+    for (int e0 = 0; e0 < d; e0 += kE) {
+      __syncthreads();  // the slice (and, at first, pq) is free / written
+#pragma unroll
+      for (int x = 0; x < kLoads; ++x) {
+        const int t = x * kSelThreads + tid, j = t / (kE / 4), a = t % (kE / 4);
+        float* dst = kt + 4 * a * kSelCols + (j ^ (a << 2));
+        dst[0] = next[x].x;
+        dst[kSelCols] = next[x].y;
+        dst[2 * kSelCols] = next[x].z;
+        dst[3 * kSelCols] = next[x].w;
+      }
+      __syncthreads();
+      if (e0 + kE < d) fetch(e0 + kE);  // in flight during this slice's products
+#pragma unroll 8
+      for (int e = 0; e < kE; ++e) {
+        const float4 kv = *reinterpret_cast<const float4*>(kt + e * kSelCols + ((cg ^ (e >> 2)) << 2));
+        const float kx[kTc] = {kv.x, kv.y, kv.z, kv.w};
+        float2 p[kTr / 2];
+        const float* prow = pq + (e0 + e) * kRows + rg * kTr;
+#pragma unroll
+        for (int r = 0; r < kTr / 2; ++r) p[r] = *reinterpret_cast<const float2*>(prow + 2 * r);
+#pragma unroll
+        for (int x = 0; x < kTc; ++x)
+#pragma unroll
+          for (int r = 0; r < kTr / 2; ++r) acc[r][x] = ffma2(p[r], make_float2(kx[x], kx[x]), acc[r][x]);
       }
     }
 #pragma unroll
-    for (int r = 0; r < kSelMaxRows; ++r)
-      if (r < rows) {
-        sc[r * nk + j0] = acc0[r];
-        if (has1) sc[r * nk + j1] = acc1[r];
+    for (int x = 0; x < kTc; ++x) {
+      const int j = j0 + cg * kTc + x;
+      if (j >= nk) continue;
+#pragma unroll
+      for (int r = 0; r < kTr / 2; ++r) {
+        const int r0 = rg * kTr + 2 * r;
+        if (r0 < rows) sc[r0 * nk + j] = acc[r][x].x;
+        if (r0 + 1 < rows) sc[(r0 + 1) * nk + j] = acc[r][x].y;
       }
+    }
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  uint32_t* hw = hist + w * 256;
+  const int lane = tid & 31, w = tid >> 5, W = (nk + 31) / 32;
   const uint32_t lt_mask = (1u << lane) - 1u;
   for (int r = w; r < rows; r += kSelThreads / 32) {
     const float* srow = sc + r * nk;
-    uint32_t prefix = 0, pmask = 0;
-    int k = k_rho;  // rank still to find among keys matching the prefix
-    for (int pass = 3; pass >= 0; --pass) {
-      const int shift = pass * 8;
-      for (int b = lane; b < 256; b += 32) hw[b] = 0;
-      __syncwarp();
+    uint32_t thr = 0;
+    int equal = 0;
+    if (W <= 8) {
+      select_row<8>(srow, nk, k_rho, lane, thr, equal);
+    } else if (W <= 16) {
+      select_row<16>(srow, nk, k_rho, lane, thr, equal);
+    } else if (W <= 24) {
+      select_row<24>(srow, nk, k_rho, lane, thr, equal);
+    } else if (W <= kSelRegKeys) {
+      select_row<kSelRegKeys>(srow, nk, k_rho, lane, thr, equal);
+    } else {
+      uint32_t lo = 0xffffffffu, hi = 0u;
       for (int j = lane; j < nk; j += 32) {
-        uint32_t u = order_key(srow[j]);
-        if ((u & pmask) == prefix) atomicAdd(&hw[(u >> shift) & 255u], 1u);
+        const uint32_t u = order_key(srow[j]);
+        lo = min(lo, u);
+        hi = max(hi, u);
       }
-      __syncwarp();
-      // lane l owns bins 255-8l .. 248-8l (descending); find the bin holding rank k.
-      uint32_t cnt[8];
-      uint32_t local = 0;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        cnt[q] = hw[255 - 8 * lane - q];
-        local += cnt[q];
-      }
-      uint32_t incl = local;
-      for (int o = 1; o < 32; o <<= 1) {
-        uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-      }
-      const uint32_t before = incl - local;
-      const bool here = before < (uint32_t)k && (uint32_t)k <= incl;
-      uint32_t digit = 0, above = 0;
-      if (here) {
-        uint32_t c = before;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          if (c + cnt[q] >= (uint32_t)k) {
-            digit = 255 - 8 * lane - q;
-            above = c;
-            break;
-          }
-          c += cnt[q];
-        }
-      }
-      const int src = __ffs(__ballot_sync(0xffffffffu, here)) - 1;
-      digit = __shfl_sync(0xffffffffu, digit, src);
-      above = __shfl_sync(0xffffffffu, above, src);
-      k -= (int)above;
-      prefix |= digit << shift;
-      pmask |= 0xFFu << shift;
-      __syncwarp();
+      lo = __reduce_min_sync(0xffffffffu, lo);
+      hi = __reduce_max_sync(0xffffffffu, hi);
+      select_kth(
+          [&](uint32_t cand) {
+            int n = 0;
+            for (int j = lane; j < nk; j += 32) n += order_key(srow[j]) >= cand;
+            return n;
+          },
+          k_rho, lo, hi, nk, thr, equal);
     }
-    // prefix = the K_rho-th largest key; take all larger keys and the first k equal ones.
+    // all keys above thr, and the first `equal` ones at it
     const int row = h * nq + i0 + r;
     int32_t* out = col_idx + (int64_t)row * k_rho;
-    uint8_t* brow = bitmap + (int64_t)row * nk;
+    uint32_t* brow = bits + (int64_t)row * W;
     int n_sel = 0, n_eq = 0;
-    for (int j0 = 0; j0 < nk; j0 += 32) {
-      const int j = j0 + lane;
-      uint32_t u = j < nk ? order_key(srow[j]) : 0u;
+    for (int x = 0; x < W; ++x) {
+      const int j = 32 * x + lane;
       const bool valid = j < nk;
-      const bool gt = valid && u > prefix;
-      const bool eq = valid && u == prefix;
-      const uint32_t eqb = __ballot_sync(0xffffffffu, eq);
-      const int eq_rank = n_eq + __popc(eqb & lt_mask);
-      const bool sel = gt || (eq && eq_rank < k);
+      const uint32_t u = valid ? order_key(srow[j]) : 0u;
+      const uint32_t eqb = __ballot_sync(0xffffffffu, valid && u == thr);
+      const bool sel = valid && (u > thr || (u == thr && n_eq + __popc(eqb & lt_mask) < equal));
       const uint32_t selb = __ballot_sync(0xffffffffu, sel);
       if (sel) out[n_sel + __popc(selb & lt_mask)] = j;
-      if (valid) brow[j] = sel ? 1 : 0;
+      if (lane == 0) brow[x] = selb;
       n_sel += __popc(selb);
       n_eq += __popc(eqb);
+    }
+    if (lane == 0) {
+      row_ptr[row] = row * k_rho;
+      if (row == H * nq - 1) row_ptr[row + 1] = (row + 1) * k_rho;
     }
   }
 }
 
-__global__ void fill_uniform_rowptr_kernel(int32_t* row_ptr, int n_rows, int k) {
-  int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r <= n_rows) row_ptr[r] = r * k;
+// grid (H, ceil(nk / 32)): the lists of 32 key blocks of one head from the bit
+// mask [H, nq, W].  Every row holds k_rho entries, so a head's entries start at
+// h * nq * k_rho, and what lies before these 32 columns is a population count
+// over the words to their left: no pass over all counts, no second launch
+// (count, scan and fill took 67 us at the 2048 canvas, this launch about 20).  A warp owns a run of
+// 32-row groups; ballots turn 32 rows x 32 columns round, lane c then holding
+// column c's rows.
+constexpr int kTransThreads = 256;
+__global__ void __launch_bounds__(kTransThreads) transpose_kernel(const uint32_t* __restrict__ bits, int H, int nq,
+                                                                  int nk, int k_rho, int32_t* __restrict__ col_ptr,
+                                                                  int32_t* __restrict__ row_idx) {
+  constexpr int kWarps = kTransThreads / 32;
+  __shared__ int32_t s_before[kWarps], s_count[kWarps][32];
+  const int W = (nk + 31) / 32, wc = blockIdx.y, h = blockIdx.x;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t* hb = bits + (int64_t)h * nq * W;
+  int before = 0;
+  for (int i = threadIdx.x; i < nq; i += kTransThreads)
+    for (int x = 0; x < wc; ++x) before += __popc(hb[(int64_t)i * W + x]);
+  before = __reduce_add_sync(0xffffffffu, before);
+  const int groups = (nq + 31) / 32, per = (groups + kWarps - 1) / kWarps;
+  const int g0 = min(groups, w * per), g1 = min(groups, g0 + per);
+  auto column = [&](int g) -> uint32_t {  // rows 32 g .. 32 g + 31 of column 32 wc + lane
+    const int i = 32 * g + lane;
+    const uint32_t word = i < nq ? hb[(int64_t)i * W + wc] : 0u;
+    uint32_t mine = 0;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {
+      const uint32_t b = __ballot_sync(0xffffffffu, (word >> c) & 1u);
+      if (lane == c) mine = b;
+    }
+    return mine;
+  };
+  int count = 0;
+  for (int g = g0; g < g1; ++g) count += __popc(column(g));
+  s_count[w][lane] = count;
+  if (lane == 0) s_before[w] = before;
+  __syncthreads();
+  int start = h * nq * k_rho, total = 0, ahead = 0;
+  for (int x = 0; x < kWarps; ++x) {
+    start += s_before[x];
+    total += s_count[x][lane];
+    if (x < w) ahead += s_count[x][lane];
+  }
+  int incl = total;  // prefix over the 32 columns
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  start += incl - total;
+  const int j = 32 * wc + lane;
+  if (w == 0 && j < nk) {
+    col_ptr[h * nk + j] = start;
+    if (h == H - 1 && j == nk - 1) col_ptr[H * nk] = start + total;
+  }
+  int32_t* out = row_idx + start + ahead;
+  for (int g = g0; g < g1; ++g) {
+    uint32_t m = column(g);
+    while (m) {
+      *out++ = 32 * g + __ffs(m) - 1;
+      m &= m - 1;
+    }
+  }
 }
 
-// One warp per line.  Line l = (h, a): a row i of [H][nq][nk] (transposed = 0)
-// or a column j (transposed = 1).
-__global__ void bitmap_count_kernel(const uint8_t* __restrict__ bm, int H, int nq, int nk, int transposed,
-                                    int32_t* __restrict__ counts) {
+// One side of the bitmap's lists: rows, or columns for the transpose.
+struct ListSide {
+  int32_t* ptr;   // [lines + 1]
+  int32_t* idx;
+};
+
+// One warp per line.  Line l = (h, a): a row i of [H][nq][nk] (blockIdx.y = 0) or
+// a column j (blockIdx.y = 1).
+__global__ void bitmap_count_kernel(const uint8_t* __restrict__ bm, int H, int nq, int nk, ListSide rows,
+                                    ListSide cols) {
+  const bool transposed = blockIdx.y == 1;
   const int n_lines = transposed ? nk : nq;
   const int line = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (line >= H * n_lines) return;
@@ -241,18 +410,19 @@ __global__ void bitmap_count_kernel(const uint8_t* __restrict__ bm, int H, int n
     c += v != 0;
   }
   for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) counts[line] = c;
+  if (lane == 0) (transposed ? cols : rows).ptr[line] = c;
 }
 
-// Single CTA exclusive scan of n counts into ptr[0..n].
-__global__ void __launch_bounds__(1024) scan_kernel(const int32_t* __restrict__ counts, int n,
-                                                    int32_t* __restrict__ ptr) {
+// Exclusive scan in place of the counts ptr[0..n) into ptr[0..n], one CTA a side.
+__global__ void __launch_bounds__(1024) scan_kernel(int n_rows, int n_cols, ListSide rows, ListSide cols) {
   __shared__ int64_t warp_tot[32];
+  const int n = blockIdx.x ? n_cols : n_rows;
+  int32_t* ptr = (blockIdx.x ? cols : rows).ptr;
   const int tid = threadIdx.x;
   const int per = (n + 1023) / 1024;
   const int a = min(n, tid * per), b = min(n, a + per);
   int64_t local = 0;
-  for (int t = a; t < b; ++t) local += counts[t];
+  for (int t = a; t < b; ++t) local += ptr[t];
   int64_t incl = local;
   const int lane = tid & 31, w = tid >> 5;
   for (int o = 1; o < 32; o <<= 1) {
@@ -265,15 +435,18 @@ __global__ void __launch_bounds__(1024) scan_kernel(const int32_t* __restrict__ 
   for (int i = 0; i < w; ++i) wpre += warp_tot[i];
   int64_t run = wpre + incl - local;
   for (int t = a; t < b; ++t) {
+    const int c = ptr[t];
     ptr[t] = (int32_t)run;
-    run += counts[t];
+    run += c;
   }
   if (tid == 1023) ptr[n] = (int32_t)(wpre + incl);
 }
 
-__global__ void bitmap_fill_kernel(const uint8_t* __restrict__ bm, int H, int nq, int nk, int transposed,
-                                   const int32_t* __restrict__ ptr, int32_t* __restrict__ out, int64_t cap,
-                                   int32_t* status) {
+__global__ void bitmap_fill_kernel(const uint8_t* __restrict__ bm, int H, int nq, int nk, ListSide rows,
+                                   ListSide cols, int64_t cap, int32_t* status) {
+  const bool transposed = blockIdx.y == 1;
+  const int32_t* ptr = (transposed ? cols : rows).ptr;
+  int32_t* out = (transposed ? cols : rows).idx;
   const int n_lines = transposed ? nk : nq;
   const int line = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (line >= H * n_lines) return;
@@ -302,10 +475,16 @@ __global__ void bitmap_fill_kernel(const uint8_t* __restrict__ bm, int H, int nq
 }
 
 // ----------------------------------------------------------------- launchers
-static int select_rows(int nk) {
-  int r = (64 * 1024) / (nk * 4);
-  r = r < 1 ? 1 : r;
-  return r > kSelMaxRows ? kSelMaxRows : r;
+template <int kRows, int kE>
+static cudaError_t launch_score_select(const float* pooled, int H, int d, int nq, int nk, int R, int k_rho,
+                                       int32_t* row_ptr, int32_t* col_idx, uint32_t* bits, cudaStream_t stream) {
+  const size_t smem = ((size_t)kRows * d + (size_t)kE * kSelCols + (size_t)R * nk) * sizeof(float);
+  cudaError_t e =
+      cudaFuncSetAttribute(score_select_kernel<kRows, kE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  score_select_kernel<kRows, kE><<<dim3(H, (nq + R - 1) / R), kSelThreads, smem, stream>>>(
+      pooled, H, d, nq, nk, R, k_rho, row_ptr, col_idx, bits);
+  return cudaGetLastError();
 }
 
 size_t block_mask_ws(const MaskProblem& p, int mode) {
@@ -317,28 +496,17 @@ size_t block_mask_ws(const MaskProblem& p, int mode) {
   return pooled + ((bitmap + 255) / 256) * 256 + counts;
 }
 
-static cudaError_t csr_from_bitmap(const uint8_t* bm, int H, int nq, int nk, int transposed, int32_t* ptr,
-                                   int32_t* out, int64_t cap, int32_t* counts, int32_t* status,
-                                   cudaStream_t stream) {
-  const int lines = H * (transposed ? nk : nq);
-  const int grid = (lines + 7) / 8;
-  if (lines == 0) return cudaSuccess;
-  bitmap_count_kernel<<<grid, 256, 0, stream>>>(bm, H, nq, nk, transposed, counts);
-  scan_kernel<<<1, 1024, 0, stream>>>(counts, lines, ptr);
-  bitmap_fill_kernel<<<grid, 256, 0, stream>>>(bm, H, nq, nk, transposed, ptr, out, cap, status);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_block_mask_topk(const MaskProblem& p, const void* q, const void* k, int k_rho, int32_t* row_ptr,
                                    int32_t* col_idx, int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap,
                                    void* ws, int32_t* status, int sms, cudaStream_t stream) {
   (void)sms;
   const int H = p.H, nq = p.nq, nk = p.nk, d = p.d;
   float* pooled = static_cast<float*>(ws);
-  uint8_t* bitmap = reinterpret_cast<uint8_t*>(pooled + (size_t)H * (nq + nk) * d);
-  size_t bm_bytes = (((size_t)H * nq * nk + 255) / 256) * 256;
-  int32_t* counts = reinterpret_cast<int32_t*>(bitmap + bm_bytes);
-  dim3 pg(nq > nk ? nq : nk, 2);
+  // bit mask: 4 ceil(nk / 32) bytes a row, within the bytes that block_mask_ws
+  // counts for the mask (nk a row) and, for nk < 4, the counts after it
+  uint32_t* bits = reinterpret_cast<uint32_t*>(pooled + (size_t)H * (nq + nk) * d);
+  const int elems = p.dtype == UT_BF16 ? 8 : 4;
+  dim3 pg(nq > nk ? nq : nk, 2, (H * d / elems + kPoolThreads - 1) / kPoolThreads);
   if (p.dtype == UT_BF16)
     block_pool_kernel<__nv_bfloat16><<<pg, kPoolThreads, 0, stream>>>(
         static_cast<const __nv_bfloat16*>(q), static_cast<const __nv_bfloat16*>(k), p.N, H, d, p.row_stride, p.block,
@@ -347,29 +515,36 @@ cudaError_t launch_block_mask_topk(const MaskProblem& p, const void* q, const vo
     block_pool_kernel<float><<<pg, kPoolThreads, 0, stream>>>(static_cast<const float*>(q),
                                                               static_cast<const float*>(k), p.N, H, d, p.row_stride,
                                                               p.block, nq, p.block_k, nk, pooled);
-  const int R = select_rows(nk);
-  size_t smem = ((size_t)R * d + (size_t)R * nk) * sizeof(float) + 8 * 256 * sizeof(uint32_t);
-  cudaError_t e = cudaFuncSetAttribute(score_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // query blocks per CTA: as many as keep their scores within 64 KB (three CTAs
+  // per SM overlap one's selection with another's products), at least one; the
+  // narrower tiles do not compute rows that a CTA does not hold, and the short
+  // slice leaves the longest rows their room
+  int R = (64 * 1024) / (nk * 4);
+  R = R < 1 ? 1 : (R > kSelRows ? kSelRows : R);
+  const bool roomy = ((size_t)4 * d + 16 * kSelCols + (size_t)R * nk) * sizeof(float) <= 232448;  // 227 KB a block
+  auto launch = R > 8 ? launch_score_select<16, 16>
+                      : (R > 4 ? launch_score_select<8, 16>
+                               : (roomy ? launch_score_select<4, 16> : launch_score_select<4, 4>));
+  const cudaError_t e = launch(pooled, H, d, nq, nk, R, k_rho, row_ptr, col_idx, bits, stream);
   if (e != cudaSuccess) return e;
-  dim3 sg(H, (nq + R - 1) / R);
-  score_select_kernel<<<sg, kSelThreads, smem, stream>>>(pooled, H, d, nq, nk, R, k_rho, col_idx, bitmap);
-  fill_uniform_rowptr_kernel<<<(H * nq + 1 + 255) / 256, 256, 0, stream>>>(row_ptr, H * nq, k_rho);
-  if (col_ptr_t && row_idx_t) {
-    e = csr_from_bitmap(bitmap, H, nq, nk, 1, col_ptr_t, row_idx_t, col_cap, counts, status, stream);
-    if (e != cudaSuccess) return e;
-  }
+  if (col_ptr_t && row_idx_t)
+    transpose_kernel<<<dim3(H, (nk + 31) / 32), kTransThreads, 0, stream>>>(bits, H, nq, nk, k_rho, col_ptr_t,
+                                                                          row_idx_t);
   return cudaGetLastError();
 }
 
 cudaError_t launch_block_mask_bitmap(const MaskProblem& p, const uint8_t* bitmap, int32_t* row_ptr, int32_t* col_idx,
-                                     int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap, void* ws,
-                                     int32_t* status, cudaStream_t stream) {
-  int32_t* counts = static_cast<int32_t*>(ws);
-  cudaError_t e = csr_from_bitmap(bitmap, p.H, p.nq, p.nk, 0, row_ptr, col_idx, col_cap, counts, status, stream);
-  if (e != cudaSuccess) return e;
-  if (col_ptr_t && row_idx_t)
-    e = csr_from_bitmap(bitmap, p.H, p.nq, p.nk, 1, col_ptr_t, row_idx_t, col_cap, counts, status, stream);
-  return e;
+                                     int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap, int32_t* status,
+                                     cudaStream_t stream) {
+  const bool with_cols = col_ptr_t && row_idx_t;
+  const ListSide rows{row_ptr, col_idx}, cols{col_ptr_t, row_idx_t};
+  const int lines = p.H * (with_cols && p.nk > p.nq ? p.nk : p.nq);
+  const dim3 grid((lines + 7) / 8, with_cols ? 2 : 1);
+  if (lines == 0) return cudaSuccess;
+  bitmap_count_kernel<<<grid, 256, 0, stream>>>(bitmap, p.H, p.nq, p.nk, rows, cols);
+  scan_kernel<<<with_cols ? 2 : 1, 1024, 0, stream>>>(p.H * p.nq, p.H * p.nk, rows, cols);
+  bitmap_fill_kernel<<<grid, 256, 0, stream>>>(bitmap, p.H, p.nq, p.nk, rows, cols, col_cap, status);
+  return cudaGetLastError();
 }
 
 }  // namespace ut

@@ -45,8 +45,8 @@ cudaError_t launch_block_mask_topk(const MaskProblem& p, const void* q, const vo
                                    int32_t* col_idx, int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap,
                                    void* ws, int32_t* status, int sms, cudaStream_t stream);
 cudaError_t launch_block_mask_bitmap(const MaskProblem& p, const uint8_t* bitmap, int32_t* row_ptr, int32_t* col_idx,
-                                     int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap, void* ws,
-                                     int32_t* status, cudaStream_t stream);
+                                     int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap, int32_t* status,
+                                     cudaStream_t stream);
 
 // attention problems
 struct AttnProblem {

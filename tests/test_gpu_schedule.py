@@ -153,3 +153,51 @@ def test_fp32_pieces_and_alignment(N, H, d, b, aligned):
     assert np.abs(got[fin] - want[fin]).max(initial=0.0) <= 1e-5
     for gg, rr, name in zip(grads, (q.grad, k.grad, v.grad), ("dQ", "dK", "dV")):
         assert np.abs(to_np(gg) - rr.cpu().numpy()).max() <= 2e-5, name
+
+
+@pytest.mark.parametrize("N,H,bq,bk,rho", [(100, 2, 128, 128, 1.0), (4000, 3, 128, 64, 0.3), (4160, 2, 32, 32, 0.1),
+                                           (5000, 1, 64, 4, 0.02), (9000, 1, 128, 2, 0.01), (129, 5, 64, 128, 0.5),
+                                           (5400, 1, 128, 2, 0.02), (50100, 1, 8192, 1, 0.001)])
+@pytest.mark.parametrize("ties", [False, True])
+def test_topk_lists_and_transpose(N, H, bq, bk, rho, ties):
+    """Top-K lists at the edges of the column tiles (N_k of 1, 33, over 1,024 and
+    over 4,096, where keys no longer fit registers and fewer rows share a CTA;
+    over 49,000, where only the short slice leaves room):
+    the scores that the lists imply are the largest, ties go to the smaller
+    index, and the transpose holds the same pairs, ascending."""
+    from paper_2609_23169_gb300 import ultratex as u
+    d = 64
+    g = np.random.Generator(np.random.PCG64([80, N]))
+    # small integers: pooled means times a power of two and their products are exact in fp32
+    q, k = (torch.from_numpy(g.integers(-2, 3, (N, H, d)).astype(np.float32) if not ties else
+                             np.repeat(g.integers(-1, 2, (N, H, 1)), d, 2).astype(np.float32)).cuda() for _ in range(2))
+    shape = u.AttnShape(N, H, d, bq, u.UT_F32, H * d, bk)
+    rp, ci, cp, ri = (t.cpu().numpy() for t in u.ut_block_mask(shape, u.UT_MASK_TOPK, q, k, rho))
+    nq, nk = -(-N // bq), -(-N // bk)
+    kr = u.ut_topk_count(rho, nk)
+    assert np.array_equal(rp, np.arange(H * nq + 1) * kr)
+    lists = ci[:H * nq * kr].reshape(H, nq, kr)
+    assert (np.diff(lists, axis=2) > 0).all() and lists.min() >= 0 and lists.max() < nk
+
+    def pool(x, b, nb):
+        s = np.zeros((H, nb, d))
+        for i in range(nb):
+            s[:, i] = x[i * b:(i + 1) * b].sum(0, dtype=np.float64) / min(b, N - i * b)
+        return s
+
+    xq, xk = q.cpu().numpy().astype(np.float64), k.cpu().numpy().astype(np.float64)
+    sc = np.einsum("hid,hjd->hij", pool(xq, bq, nq), pool(xk, bk, nk))
+    keep = np.zeros(sc.shape, bool)
+    np.put_along_axis(keep, lists, True, 2)
+    worst_in = np.where(keep, sc, np.inf).min(2)
+    best_out = np.where(keep, -np.inf, sc).max(2)
+    eps = 1e-4 * np.abs(sc).max()  # fp32 scores against 64 bits
+    assert (worst_in >= best_out - eps).all()
+    if not ties:
+        order = np.argsort(-sc, axis=2, kind="stable")[:, :, :kr]
+        clear = (worst_in - best_out > eps)
+        want = np.sort(order, axis=2)
+        assert np.array_equal(lists[clear], want[clear])
+    pairs = np.argwhere(keep.transpose(0, 2, 1))
+    assert np.array_equal(cp, np.concatenate([[0], np.cumsum(keep.sum(1).reshape(-1))]))
+    assert np.array_equal(ri[:len(pairs)], pairs[:, 2])
