@@ -2,8 +2,8 @@
 // path for fp32 inputs, whose tolerance rules out tf32 tensor cores.
 //
 //   attn_bwd_pre_kernel  D_r = dO_r . O_r.
-//   attn_f32_kernel      one CTA per 32 own rows of a head, walking the rows of
-//                        the other side that its block lists:
+//   attn_*_f32_kernel    a cluster of two CTAs per 32 own rows of a head, walking
+//                        the rows of the other side that its block lists:
 //     kFwd   own Q, other K, V: online softmax; O, LSE.
 //     kDq    own Q, dO, other K, V: dQ_r = scale * sum_k P_rk (dO_r . V_k - D_r) K_k.
 //     kDkv   own K, V, other Q, dO over the transposed lists (query blocks that
@@ -16,15 +16,17 @@
 // 128 threads in 4 x 4 (D = 128: 4 x 2) register tiles, so that eight 16-byte
 // shared loads feed 64 FMAs, two to an instruction (even and odd d summed
 // apart), and the tile goes through shared memory to the second product.  The
-// CTA's two groups of 128 threads take alternate chunks of the list (few own
-// tiles exist at these sizes, so the list is what is left to split) and add
-// their sums at the end; each group copies its next chunk with cp.async while
+// two groups of 128 threads in each of the cluster's CTAs take chunks of the list
+// in turn (few own tiles exist at these sizes and some lists are far longer than
+// the others, so the list is what is left to split) and add their sums at the
+// end, across the CTAs through distributed shared memory; each group copies its next chunk with cp.async while
 // it works on the present one.  The row maximum is updated once per chunk, not
 // per key.
 // Measured: forward and backward of 2,002 tokens, 2 heads, D = 64, 32-row blocks
-// 8,746 -> 243 us (45 forward, 193 backward; the longest lists, 63 blocks, set
-// the backward's time); the whole path over 195 tokens 1,414 -> 233 us.  Errors
-// against 64 bits 4.7e-7 (7.2e-7 before: fewer rescalings and shorter chains).
+// 8,746 -> 243 us with one CTA per tile (45 forward, 193 backward), 201 with two
+// (47, 150); the whole path over 195 tokens 1,414 -> 233 -> 168 us, the last with
+// less host work.  Errors against 64 bits 7.2e-7 -> 4.0e-7 (fewer rescalings,
+// shorter chains).
 #include <math.h>
 
 #include "common.cuh"
@@ -33,7 +35,8 @@
 namespace ut {
 
 constexpr int kOwn = 32;          // own rows per CTA
-constexpr int kGroups = 2;        // thread groups, alternate chunks of the list
+constexpr int kGroups = 2;        // thread groups of a CTA
+constexpr int kParts = 2;         // CTAs of a cluster: kGroups * kParts groups share the list
 constexpr int kGroupThreads = 128;
 constexpr int kF32Threads = kGroups * kGroupThreads;
 
@@ -79,6 +82,19 @@ UT_DEV void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 UT_DEV void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+// Address of the same shared variable in CTA `rank` of the cluster, a store
+// there, and the cluster's barrier (release / acquire).
+UT_DEV uint32_t cluster_addr(const void* p, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+UT_DEV void st_cluster(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+UT_DEV void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 UT_DEV void group_sync(int g) { asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(kGroupThreads) : "memory"); }
 
@@ -189,10 +205,12 @@ UT_DEV void store_rows(float* out, int64_t r0, int valid, int64_t off, int64_t r
 }
 
 template <int D, int MODE, bool kVec>
-UT_DEV void f32_tile(const F32Args& a, F32Smem<D, MODE>& sm) {
+UT_DEV void f32_tile(const F32Args& a, F32Smem<D, MODE>& sm, int part) {
   using S = F32Smem<D, MODE>;
   constexpr int KC = S::KC, NX = KC / 16, LP = S::LP, NC = D / 32, kSubs = KC / 32;
   const int g = threadIdx.x / kGroupThreads, t = threadIdx.x % kGroupThreads;
+  const int gg = part * kGroups + g;  // this group among all that share the list
+  constexpr int kAll = kGroups * kParts;
   const int rg = t / 16, c = t % 16;  // rows rg * 4 .. + 3; columns c + 16 x of the scores, c * 4 .. of the outputs
   const int h = blockIdx.y;
   const int64_t r0 = (int64_t)blockIdx.x * kOwn, off = (int64_t)h * D;
@@ -232,7 +250,7 @@ UT_DEV void f32_tile(const F32Args& a, F32Smem<D, MODE>& sm) {
   copy_rows<D, kVec>(sm.a1, own1, r0, valid, kOwn, off, a.rs, threadIdx.x, kF32Threads);
   if (MODE != kFwd) copy_rows<D, kVec>(sm.a2, own2, r0, valid, kOwn, off, a.rs, threadIdx.x, kF32Threads);
   cp_commit();
-  if (g < chunks) load(g, 0);
+  if (gg < chunks) load(gg, 0);
   cp_commit();
   cp_wait<1>();
   __syncthreads();
@@ -254,8 +272,8 @@ UT_DEV void f32_tile(const F32Args& a, F32Smem<D, MODE>& sm) {
     d_r[y] = MODE == kDq && r < valid ? a.dsum[(int64_t)h * a.N + r0 + r] : 0.f;
   }
   int stage = 0;
-  for (int ch = g; ch < chunks; ch += kGroups, stage ^= 1) {
-    if (ch + kGroups < chunks) load(ch + kGroups, stage ^ 1);
+  for (int ch = gg; ch < chunks; ch += kAll, stage ^= 1) {
+    if (ch + kAll < chunks) load(ch + kAll, stage ^ 1);
     cp_commit();
     cp_wait<1>();
     group_sync(g);
@@ -324,65 +342,79 @@ UT_DEV void f32_tile(const F32Args& a, F32Smem<D, MODE>& sm) {
     if constexpr (MODE == kDkv) accumulate<D>(sm.g[g].ds, st.b1, rg, c, acc2);
     group_sync(g);  // this stage and the tile are free for the chunk after the next
   }
-  // the other groups' sums, through the first group's stages (no copy is in flight)
+  // the groups' sums: the second group's through the first one's stages, then
+  // the second CTA's through the second group's stages of the first CTA (no copy
+  // is in flight in either)
   cp_wait<0>();
-  __syncthreads();
   constexpr int kVals = 4 * NC * 2 * (MODE == kDkv ? 2 : 1) + 8;
   static_assert(kVals * kGroupThreads * sizeof(float) <= sizeof(typename S::Stage) * 2, "merge area");
-  float* ex = reinterpret_cast<float*>(&sm.g[0].st[0]) + t;
+  static_assert(kGroups == 2 && kParts == 2, "each merge adds one to the other");
   if constexpr (MODE == kFwd) {
 #pragma unroll
     for (int y = 0; y < 4; ++y)
 #pragma unroll
       for (int w = 8; w; w >>= 1) l[y] += __shfl_xor_sync(0xffffffffu, l[y], w);
   }
-  static_assert(kGroups == 2, "the merge adds one group to the other");
-  if (g == 1) {
+  auto give = [&](auto put) {  // put(n, value)
     int n = 0;
 #pragma unroll
     for (int y = 0; y < 4; ++y)
 #pragma unroll
       for (int x = 0; x < NC; ++x) {
-        ex[n++ * kGroupThreads] = acc[y][x].x;
-        ex[n++ * kGroupThreads] = acc[y][x].y;
+        put(n++, acc[y][x].x);
+        put(n++, acc[y][x].y);
         if (MODE == kDkv) {
-          ex[n++ * kGroupThreads] = acc2[y][x].x;
-          ex[n++ * kGroupThreads] = acc2[y][x].y;
+          put(n++, acc2[y][x].x);
+          put(n++, acc2[y][x].y);
         }
       }
 #pragma unroll
     for (int y = 0; y < 4; ++y) {
-      ex[n++ * kGroupThreads] = m[y];
-      ex[n++ * kGroupThreads] = l[y];
+      put(n++, m[y]);
+      put(n++, l[y]);
     }
-  }
-  __syncthreads();
-  if (g != 0) return;
-  float f0[4], f1[4];
+  };
+  auto add = [&](const float* ex) {
+    float f0[4], f1[4];
 #pragma unroll
-  for (int y = 0; y < 4; ++y) {
-    f0[y] = f1[y] = 1.f;
-    if (MODE == kFwd) {
-      const float mo = ex[(4 * NC * 2 + 2 * y) * kGroupThreads], lo = ex[(4 * NC * 2 + 2 * y + 1) * kGroupThreads];
-      const float mn = fmaxf(m[y], mo), ref = mn == -INFINITY ? 0.f : mn;
-      f0[y] = expf(m[y] - ref);
-      f1[y] = expf(mo - ref);
-      l[y] = l[y] * f0[y] + lo * f1[y];
-      m[y] = mn;
-    }
-  }
-  int n = 0;
-#pragma unroll
-  for (int y = 0; y < 4; ++y)
-#pragma unroll
-    for (int x = 0; x < NC; ++x) {
-      acc[y][x].x = acc[y][x].x * f0[y] + ex[n++ * kGroupThreads] * f1[y];
-      acc[y][x].y = acc[y][x].y * f0[y] + ex[n++ * kGroupThreads] * f1[y];
-      if (MODE == kDkv) {
-        acc2[y][x].x += ex[n++ * kGroupThreads];
-        acc2[y][x].y += ex[n++ * kGroupThreads];
+    for (int y = 0; y < 4; ++y) {
+      f0[y] = f1[y] = 1.f;
+      if (MODE == kFwd) {
+        const float mo = ex[(4 * NC * 2 + 2 * y) * kGroupThreads], lo = ex[(4 * NC * 2 + 2 * y + 1) * kGroupThreads];
+        const float mn = fmaxf(m[y], mo), ref = mn == -INFINITY ? 0.f : mn;
+        f0[y] = expf(m[y] - ref);
+        f1[y] = expf(mo - ref);
+        l[y] = l[y] * f0[y] + lo * f1[y];
+        m[y] = mn;
       }
     }
+    int n = 0;
+#pragma unroll
+    for (int y = 0; y < 4; ++y)
+#pragma unroll
+      for (int x = 0; x < NC; ++x) {
+        acc[y][x].x = acc[y][x].x * f0[y] + ex[n++ * kGroupThreads] * f1[y];
+        acc[y][x].y = acc[y][x].y * f0[y] + ex[n++ * kGroupThreads] * f1[y];
+        if (MODE == kDkv) {
+          acc2[y][x].x += ex[n++ * kGroupThreads];
+          acc2[y][x].y += ex[n++ * kGroupThreads];
+        }
+      }
+  };
+  float* ex0 = reinterpret_cast<float*>(&sm.g[0].st[0]) + t;
+  float* ex1 = reinterpret_cast<float*>(&sm.g[1].st[0]) + t;
+  __syncthreads();
+  if (g == 1) give([&](int n, float v) { ex0[n * kGroupThreads] = v; });
+  __syncthreads();
+  if (g == 0) add(ex0);
+  cluster_sync();  // the first CTA's second group is done with its stages
+  if (part == 1 && g == 0) {
+    const uint32_t to = cluster_addr(ex1, 0);
+    give([&](int n, float v) { st_cluster(to + n * kGroupThreads * (uint32_t)sizeof(float), v); });
+  }
+  cluster_sync();
+  if (part != 0 || g != 0) return;
+  add(ex1);
   float f[4];
 #pragma unroll
   for (int y = 0; y < 4; ++y) f[y] = MODE == kFwd ? (l[y] > 0.f ? 1.f / l[y] : 0.f) : 1.f;
@@ -396,19 +428,23 @@ UT_DEV void f32_tile(const F32Args& a, F32Smem<D, MODE>& sm) {
   }
 }
 
-// grid (own tiles, H)
+// grid (own tiles, H, kParts): a cluster spans z
 template <int D>
-__global__ void __launch_bounds__(kF32Threads, 1) attn_fwd_f32_kernel(const F32Args a) {
+__global__ void __cluster_dims__(1, 1, kParts) __launch_bounds__(kF32Threads, 1)
+    attn_fwd_f32_kernel(const F32Args a) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
-  f32_tile<D, kFwd, true>(a, *reinterpret_cast<F32Smem<D, kFwd>*>(smem_raw));
+  f32_tile<D, kFwd, true>(a, *reinterpret_cast<F32Smem<D, kFwd>*>(smem_raw), blockIdx.z);
 }
 
-// grid (own tiles, H, 2): z = 0 the query tiles (dQ), z = 1 the key tiles (dK, dV)
+// grid (own tiles, H, 2 kParts): the first kParts of z the query tiles (dQ), the
+// others the key tiles (dK, dV)
 template <int D, bool kVec>
-__global__ void __launch_bounds__(kF32Threads, 1) attn_bwd_f32_kernel(const F32Args dq, const F32Args dkv) {
+__global__ void __cluster_dims__(1, 1, kParts) __launch_bounds__(kF32Threads, 1)
+    attn_bwd_f32_kernel(const F32Args dq, const F32Args dkv) {
   extern __shared__ __align__(16) uint8_t smem_raw[];
-  if (blockIdx.z == 0) f32_tile<D, kDq, kVec>(dq, *reinterpret_cast<F32Smem<D, kDq>*>(smem_raw));
-  else f32_tile<D, kDkv, kVec>(dkv, *reinterpret_cast<F32Smem<D, kDkv>*>(smem_raw));
+  const int part = blockIdx.z % kParts;
+  if (blockIdx.z < kParts) f32_tile<D, kDq, kVec>(dq, *reinterpret_cast<F32Smem<D, kDq>*>(smem_raw), part);
+  else f32_tile<D, kDkv, kVec>(dkv, *reinterpret_cast<F32Smem<D, kDkv>*>(smem_raw), part);
 }
 
 // D_r = dO_r . O_r: 16 lanes per (row, head)
@@ -434,7 +470,7 @@ static cudaError_t fwd_impl(const AttnProblem& p, const F32Args& a, cudaStream_t
   constexpr size_t smem = sizeof(F32Smem<D, kFwd>);
   cudaError_t e = cudaFuncSetAttribute(attn_fwd_f32_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  attn_fwd_f32_kernel<D><<<dim3((unsigned)((p.N + kOwn - 1) / kOwn), p.H), kF32Threads, smem, s>>>(a);
+  attn_fwd_f32_kernel<D><<<dim3((unsigned)((p.N + kOwn - 1) / kOwn), p.H, kParts), kF32Threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -474,7 +510,7 @@ static cudaError_t bwd_impl(const AttnProblem& p, const F32Args& dq, const F32Ar
       cudaFuncSetAttribute(attn_bwd_f32_kernel<D, kVec>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   attn_bwd_f32_kernel<D, kVec>
-      <<<dim3((unsigned)((p.N + kOwn - 1) / kOwn), p.H, 2), kF32Threads, smem, s>>>(dq, dkv);
+      <<<dim3((unsigned)((p.N + kOwn - 1) / kOwn), p.H, 2 * kParts), kF32Threads, smem, s>>>(dq, dkv);
   return cudaGetLastError();
 }
 
