@@ -466,7 +466,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
           if (!(ok = next_item(kk, w, false)) || w < 0) break;
           BlockSteps<kMode> tl;
           tl.init(prm.ptr, prm.idx, w / prm.nq, w % prm.nq, prm.nk_fine, prm.k_rows_per_tile, prm.list_shift);
-          const int L = tl.count_warp();
+          const int L = uniform(tl.count_warp());
           if (L <= 0) continue;
           if (!(ok = warp_wait(&sm.kv_full, ki & 1, abort_flag, prm.status, prm.timeout_ns))) break;
           auto issue_st = [&](int t) -> bool {  // S^T_t = K Q_t^T into R0
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
       const int h = w / prm.nq, j = w % prm.nq;
       BlockSteps<kMode> tl;
       tl.init(prm.ptr, prm.idx, h, j, prm.nk_fine, prm.k_rows_per_tile, prm.list_shift);
-      const int L = tl.count_warp();
+      const int L = uniform(tl.count_warp());
       const int64_t gk = (int64_t)j * kTile + krow;
       const bool row_ok = gk < prm.N;
       __nv_bfloat16* dv_row = prm.out0 + gk * prm.rs + (int64_t)h * D + half * HD;
@@ -738,7 +738,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
       const int h = w / prm.nq;
       BlockSteps<kMode> tl;
       tl.init(prm.ptr, prm.idx, h, w % prm.nq, prm.nk_fine, prm.k_rows_per_tile, prm.list_shift);
-      const int L = tl.count_warp();
+      const int L = uniform(tl.count_warp());
       if (L <= 0) continue;
       for (int t = 0; t < L; ++t) {
         const uint32_t qd = qd0 + t;
