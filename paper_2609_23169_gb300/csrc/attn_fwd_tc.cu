@@ -70,6 +70,26 @@ constexpr int kStages = 3;                       // K and V ring depth
 constexpr uint32_t kTileChunkBytes = 128 * 128;  // 128 rows x 128 bytes (64 bf16)
 constexpr uint32_t kColO = 256, kColQ = 384;     // TMEM column bases (Q: two buffers of 64 columns)
 
+// Static schedule of lists of unequal length.  Dealt out in index order, round
+// by round, the busiest of 152 CTAs has 244 steps against a mean of 199 at the
+// 512 canvas (structured lists, reference kept in full) and up to 1.8 times the
+// mean on smaller ones.  The entry point has no workspace for a common counter
+// or order, so every CTA computes the same order for itself, in its still unused
+// K ring: items by length, longest first, equal ones by index, dealt out
+// boustrophedon (202 steps there).  Only where it pays: a few items per CTA
+// (the more there are the better index order evens out), K and V of all heads in
+// L2 at once (the order gives up that neighbours share a head: with 43 MB a head
+// an order across heads costs 31%), index order at least 5% off the mean, and
+// 128-row blocks on both sides.  512 canvas: 219 -> 207 us.
+constexpr int kSortItems = 4096, kSortBins = 1024, kSortRounds = 32;
+constexpr int64_t kSortKvBytes = 96ll << 20;
+struct FwdSort {
+  uint16_t length[kSortItems];
+  uint16_t bin[kSortItems];  // 0: the longest
+  int32_t start[kSortBins];  // entries per bin, then the rank of its first item
+  int32_t longest, busiest, total;
+};
+
 template <int D>
 struct FwdSmem {
   static constexpr int kChunks = D / 64;
@@ -90,6 +110,7 @@ struct FwdSmem {
   uint64_t o_empty, mma_done;
   uint64_t m_full[2][4];       // [tile & 1][lane quarter]: row maxima published
   uint64_t l_full[2][4];       // [item & 1][lane quarter]: the other warpgroup's normalisers
+  int32_t mine[kSortRounds];   // this CTA's items, where they are sorted
   float m_row[2][kBM];         // row maximum used by tile (tile & 1)
   float l_row[2][kBM];         // normaliser handed over, per item & 1
   uint32_t tmem_base;
@@ -113,7 +134,80 @@ struct FwdParams {
   uint64_t timeout_ns;
 };
 
-template <int D, int kMode>
+// Fills mine[] with this CTA's items, longest first over all CTAs; false (in
+// every CTA alike) if index order is even enough.  All threads call it.
+UT_DEV bool sort_items(const FwdParams& prm, FwdSort& st, int32_t* mine) {
+  const int n = prm.n_items, G = gridDim.x, tid = threadIdx.x;
+  if (tid == 0) st.longest = st.busiest = st.total = 0;
+  for (int b = tid; b < kSortBins; b += kFwdThreads) st.start[b] = 0;
+  __syncthreads();
+  int mx = 0;
+  for (int x = tid; x < n; x += kFwdThreads) {  // listed blocks of item x
+    const int len = min(65535, prm.row_ptr[x + 1] - prm.row_ptr[x]);
+    st.length[x] = (uint16_t)len;
+    mx = max(mx, len);
+  }
+  atomicMax(&st.longest, mx);
+  __syncthreads();
+  for (int b = tid; b < G; b += kFwdThreads) {
+    int sum = 0;
+    for (int x = b; x < n; x += G) sum += st.length[x];
+    atomicMax(&st.busiest, sum);
+    atomicAdd(&st.total, sum);
+  }
+  __syncthreads();
+  if ((int64_t)st.busiest * G * 20 <= (int64_t)st.total * 21) return false;
+  const uint32_t longest = (uint32_t)max(1, st.longest);
+  for (int x = tid; x < n; x += kFwdThreads) {
+    const uint32_t b = (kSortBins - 1) - st.length[x] * (uint32_t)(kSortBins - 1) / longest;
+    st.bin[x] = (uint16_t)b;
+    atomicAdd(&st.start[b], 1);
+  }
+  __syncthreads();
+  const int lane = tid & 31;
+  if (tid < 32) {  // exclusive prefix, 32 bins a lane
+    int c[kSortBins / 32], local = 0;
+#pragma unroll
+    for (int e = 0; e < kSortBins / 32; ++e) {
+      c[e] = st.start[lane * (kSortBins / 32) + e];
+      local += c[e];
+    }
+    int run = local;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, run, o);
+      if (lane >= o) run += v;
+    }
+    run -= local;
+#pragma unroll
+    for (int e = 0; e < kSortBins / 32; ++e) {
+      st.start[lane * (kSortBins / 32) + e] = run;
+      run += c[e];
+    }
+  }
+  __syncthreads();
+  for (int k = tid >> 5; k < kSortRounds; k += kFwdThreads / 32) {  // a warp finds the item of one round
+    int rank = k * G + (k & 1 ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
+    if (rank >= n) continue;
+    int lo = 0, hi = kSortBins - 1;  // the last bin that starts at or before the rank
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (st.start[mid] <= rank) lo = mid;
+      else hi = mid - 1;
+    }
+    rank -= st.start[lo];
+    for (int x0 = 0; x0 < n; x0 += 32) {
+      const uint32_t m = __ballot_sync(0xffffffffu, x0 + lane < n && st.bin[x0 + lane] == lo);
+      if (rank < __popc(m)) {
+        if ((m >> lane & 1u) && __popc(m & ((1u << lane) - 1u)) == rank) mine[k] = x0 + lane;
+        break;
+      }
+      rank -= __popc(m);
+    }
+  }
+  return true;
+}
+
+template <int D, int kMode, bool kSort>  // kSort: sizes allow the sorted schedule
 __global__ void __launch_bounds__(kFwdThreads, 1)
     attn_fwd_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_k64,
@@ -168,12 +262,38 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     tmem_alloc(&sm.tmem_base, 512);
     tmem_relinquish();
   }
+  const int G = gridDim.x;
+  bool sorted = false;
+  if constexpr (kSort) {
+    const int in_order = !sort_items(prm, *reinterpret_cast<FwdSort*>(&sm.k[0][0]), sm.mine);
+    fence_proxy_async_smem();  // the K ring is written by TMA next
+    sorted = uniform(in_order) == 0;
+  }
+  // this CTA's items: first_item(k), then next_item(w, k) until n_items or more
+  auto item_at = [&](int k) -> int {
+    if (!sorted) return blockIdx.x + k * G;
+    return k * G + (k & 1 ? G - 1 - (int)blockIdx.x : (int)blockIdx.x) < prm.n_items && k < kSortRounds ? sm.mine[k]
+                                                                                                        : prm.n_items;
+  };
+  auto first_item = [&](int& k) -> int {
+    k = 0;
+    if constexpr (kSort) return item_at(0);
+    else return blockIdx.x;
+  };
+  auto next_item = [&](int w, int& k) -> int {
+    if constexpr (kSort) return item_at(++k);
+    else return w + G;
+  };
+  // with items from shared memory the compiler has to be told what is uniform
+  auto same = [](auto x) {
+    if constexpr (kSort) return uniform(x);
+    else return x;
+  };
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
 
-  const int G = gridDim.x;
   if (warp < 4) {
   setmaxnreg_dec<kFwdRegCtl>();
   if (warp == 0) {
@@ -200,7 +320,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       const void* tmap64 = is_k ? static_cast<const void*>(&tm_k64) : static_cast<const void*>(&tm_v64);
       uint32_t qi = 0, kv = 0;
       bool ok = true;
-      for (int w = blockIdx.x; w < prm.n_items && ok; w += G) {
+      int k;
+      for (int w = first_item(k); w < prm.n_items && ok; w = next_item(w, k)) {
         const int h = w / prm.nq, i = w % prm.nq;
         BlockSteps<kMode> tl;
         tl.init(prm.row_ptr, prm.col_idx, h, i, prm.nq_fine, prm.q_rows_per_tile, prm.list_shift);
@@ -252,9 +373,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     uint32_t qi = 0, oi = 0;  // items: S started, P V started
     uint32_t firsts = 0;      // bit (tile & 3): the tile is the first of its item
     bool ok = true;
-    // item of the S cursor: index, tiles, next tile; the list bounds of the
+    // item of the S cursor: index, round, tiles, next tile; the list bounds of the
     // following item are loaded an item ahead (128-row blocks)
-    int cw = blockIdx.x, cL = 0, ct = 0;
+    int ck, cw = same(first_item(ck)), cL = 0, ct = 0;
     int n_lo = 0, n_hi = 0;
     auto load_bounds = [&](int w) {
       if (kMode == 0 && w < prm.n_items) {
@@ -263,17 +384,18 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       }
     };
     auto count_from = [&]() {  // cw, cL: the first item from cw on that lists something (cL = 0: none)
-      for (cL = 0; cw < prm.n_items; cw += G) {
+      for (cL = 0; same(cw < prm.n_items); cw = same(next_item(cw, ck))) {
         if (kMode == 0) {
-          cL = n_hi - n_lo;
-          load_bounds(cw + G);
+          cL = same(n_hi - n_lo);
+          int k = ck;
+          load_bounds(same(next_item(cw, k)));
         } else {
           BlockSteps<kMode> tl;
           tl.init(prm.row_ptr, prm.col_idx, cw / prm.nq, cw % prm.nq, prm.nq_fine, prm.q_rows_per_tile,
                   prm.list_shift);
           cL = tl.count_warp();
         }
-        if (cL > 0) return;
+        if (same(cL > 0)) return;
       }
       cL = 0;
     };
@@ -281,9 +403,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       return warp_wait(&sm.k_full[sc % kStages], (sc / kStages) & 1, abort_flag, prm.status, prm.timeout_ns);
     };
     auto issue_s = [&]() -> bool {
+      sc = same((int)sc);
+      qi = same((int)qi);
       const uint32_t st = sc % kStages, sb = sc & 1;
-      if (ct == 0 && !warp_wait(&sm.qt_full[qi & 1], (qi >> 1) & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
-      if (sc < 2 && !wait_k()) return false;
+      const bool first = same(ct == 0);
+      if (first && !warp_wait(&sm.qt_full[qi & 1], (qi >> 1) & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
+      if (same(sc < 2) && !wait_k()) return false;
       tc_fence_after();
       const uint32_t k_addr = smem_u32(sm.k[st]);
       const uint32_t q_col = tmem + kColQ + (qi & 1) * 64;
@@ -294,10 +419,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       }
       mma_commit_w(&sm.s_full[sb]);
       mma_commit_w(&sm.k_empty[st]);
-      firsts = (firsts & ~(1u << (sc & 3))) | ((ct == 0 ? 1u : 0u) << (sc & 3));
+      firsts = (firsts & ~(1u << (sc & 3))) | ((first ? 1u : 0u) << (sc & 3));
       ++sc;
-      if (++ct == cL) {
-        cw += G;
+      if (same(++ct == cL)) {
+        cw = same(next_item(cw, ck));
         ct = 0;
         ++qi;
         count_from();
@@ -305,8 +430,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       return true;
     };
     auto issue_pv = [&]() -> bool {
+      pc = same((int)pc);
       const uint32_t st = pc % kStages, n = pc / kStages, sb = pc & 1, ph = (pc >> 1) & 1;
-      const bool first = (firsts >> (pc & 3)) & 1u;
+      const bool first = same(((firsts >> (pc & 3)) & 1u) != 0);
       if (!warp_wait(&sm.v_full[st], n & 1, abort_flag, prm.status, prm.timeout_ns)) return false;
       if (first) {  // O is free once the previous item's was read
         if (!warp_wait(&sm.o_empty, (oi & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns)) return false;
@@ -314,7 +440,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       }
       // K of the S tile that follows: ready long before P, and waited for here
       // it does not stand between P V and S
-      if (cL > 0 && !wait_k()) return false;
+      if (same(cL > 0) && !wait_k()) return false;
       const uint32_t v_addr = smem_u32(sm.v[st]);
 #pragma unroll
       for (int hc = 0; hc < 2; ++hc) {
@@ -332,10 +458,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
     };
     load_bounds(cw);
     count_from();
-    for (int x = 0; x < 2 && ok && cL > 0; ++x) ok = issue_s();
-    while (ok && pc < sc) {
+    for (int x = 0; x < 2 && same(ok && cL > 0); ++x) ok = issue_s();
+    while (same(ok && pc < sc)) {
       if (!(ok = issue_pv())) break;
-      if (cL > 0) ok = issue_s();
+      if (same(cL > 0)) ok = issue_s();
     }
     // Drain: all MMAs issued by this warp complete before TMEM is freed.
     mma_commit_w(&sm.mma_done);
@@ -380,11 +506,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       }
       return true;
     };
-    for (int w = blockIdx.x; w < prm.n_items && ok; w += G) {
+    int k;
+    for (int w = same(first_item(k)); w < prm.n_items && ok; w = same(next_item(w, k))) {
       const int h = w / prm.nq, i = w % prm.nq;
       BlockSteps<kMode> tl;
       tl.init(prm.row_ptr, prm.col_idx, h, i, prm.nq_fine, prm.q_rows_per_tile, prm.list_shift);
-      const int L = tl.count_warp();
+      const int L = same(tl.count_warp());
       const int64_t grow = (int64_t)i * kBM + row;
       const bool row_ok = grow < prm.N;
       __nv_bfloat16* orow = prm.o + grow * prm.rs + (int64_t)h * D;
@@ -596,22 +723,23 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
 }
 
 static_assert(sizeof(FwdSmem<128>) <= 232448, "forward shared layout exceeds the per-block limit");
+static_assert(sizeof(FwdSort) <= kStages * FwdSmem<64>::kKVBytes, "the sort's scratch must fit the K ring");
 
-template <int D, int kMode>
+template <int D, int kMode, bool kSort = false>
 static cudaError_t launch_d(const AttnProblem& p, const CUtensorMap& tq, const CUtensorMap& tk,
                             const CUtensorMap& tv, const CUtensorMap& tk64, const CUtensorMap& tv64,
                             const FwdParams& prm, int grid, cudaStream_t stream) {
   const size_t smem = sizeof(FwdSmem<D>);
   cudaError_t e =
-      cudaFuncSetAttribute(attn_fwd_tc_kernel<D, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(attn_fwd_tc_kernel<D, kMode, kSort>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   // the setmaxnreg split assumes exactly kFwdRegLaunch registers per thread at
   // launch: with fewer, the increases would wait for registers that never come
   cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, attn_fwd_tc_kernel<D, kMode>);
+  e = cudaFuncGetAttributes(&fa, attn_fwd_tc_kernel<D, kMode, kSort>);
   if (e != cudaSuccess) return e;
   if (fa.numRegs != kFwdRegLaunch) return cudaErrorInvalidConfiguration;
-  attn_fwd_tc_kernel<D, kMode><<<grid, kFwdThreads, smem, stream>>>(tq, tk, tv, tk64, tv64, prm);
+  attn_fwd_tc_kernel<D, kMode, kSort><<<grid, kFwdThreads, smem, stream>>>(tq, tk, tv, tk64, tv64, prm);
   return cudaGetLastError();
 }
 
@@ -651,9 +779,12 @@ cudaError_t launch_attn_fwd_tc(const AttnProblem& p, const void* q, const void* 
   prm.scale_log2 = p.scale * 1.4426950408889634f;
   prm.timeout_ns = timeout_ns;
   const int grid = n_items < sms ? n_items : sms;
+  const bool sort = mode == 0 && n_items > grid && n_items <= kSortItems && n_items <= kSortRounds * grid &&
+             (int64_t)p.H * p.N * p.d * 4 <= kSortKvBytes;
 #define UT_FWD_LAUNCH(DD, MM) launch_d<DD, MM>(p, tq, tk, tv, tk64, tv64, prm, grid, stream)
 #define UT_FWD_MODES(DD)                                                                    \
-  (mode == 0 ? UT_FWD_LAUNCH(DD, 0)                                                         \
+  (sort ? launch_d<DD, 0, true>(p, tq, tk, tv, tk64, tv64, prm, grid, stream)               \
+   : mode == 0 ? UT_FWD_LAUNCH(DD, 0)                                                       \
              : (mode == 1 ? UT_FWD_LAUNCH(DD, 1) : (mode == 2 ? UT_FWD_LAUNCH(DD, 2) : UT_FWD_LAUNCH(DD, 3))))
   if (p.d == 64) return UT_FWD_MODES(64);
   return UT_FWD_MODES(128);
