@@ -700,9 +700,10 @@ def time_mask_from_alpha(w, dev, hbm_peak: float, reps: int = 20) -> dict:
 
 
 def hp_launches(hp) -> int:
-    """Kernel launches of one HotPath.step (compaction 3, Top-K lists 3 + transpose 3,
-    forward 1, backward 3 (preprocess, fused dK/dV/dQ, dQ finalize), scatter 2)."""
-    return 3 + 6 + 1 + 3 + 2
+    """Kernel launches of one HotPath.step (compaction 3, Top-K lists 3 (pool, score and
+    select, transpose), forward 1, backward 3 (preprocess, fused dK/dV/dQ, dQ finalize),
+    scatter 2)."""
+    return 3 + 3 + 1 + 3 + 2
 
 
 # ------------------------------------------------------------------- oracle

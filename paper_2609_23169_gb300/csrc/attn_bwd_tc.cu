@@ -5,9 +5,10 @@
 //   dV = P^T dO,   dS = P o (dO V^T - D),   dQ = scale * dS K,   dK = scale * dS^T Q
 // over the retained block pairs only:
 //
-//   bwd_pre_kernel          D_r and LSE_r * log2(e) per (head, row) into a
-//                           padded [H, N_t*128] workspace (padding rows: D = 0,
-//                           LSE = +inf so that they contribute P = 0).
+//   bwd_pre_kernel          -D_r and -LSE_r * log2(e) per (head, row) into a
+//                           padded [H, N_t*128] workspace (padding rows: 0 and
+//                           -inf so that they contribute P = 0), the dQ
+//                           accumulator cleared, the order of the items.
 //   bwd_fused_kernel        item (h, 128-row key tile j) over the transposed
 //                           lists: S^T and dP^T once per pair, dK and dV
 //                           accumulated in TMEM, dQ^T partials added into an
@@ -205,7 +206,7 @@ UT_DEV void tmem_ld64(uint32_t taddr, uint32_t* r) {
 // A final kernel scales the accumulator by the softmax scale and writes dQ in
 // bf16.  Roles (512 threads, four warpgroups; the register file is rebalanced
 // with setmaxnreg): warpgroup 0 = warp 0 TMA, warp 1 TMEM owner + MMA issuer
-// (warps 2-3 idle); warpgroups 1-2 = 8 elementwise warps; warpgroup 3 = 4 dQ
+// and warp 2 lane 0 the row vectors; warpgroups 1-2 = 8 elementwise warps; warpgroup 3 = 4 dQ
 // drain warps.
 // TMEM columns: R0 [0,128), RQ [128,256), dV [256,256+d), dK [384,384+d).
 // For d = 64 the A operand K^T of the dQ product is padded to 128 rows with a
@@ -223,10 +224,9 @@ constexpr uint32_t kColR0 = 0, kColRQ = 128, kColFuDv = 256, kColFuDk = 384;
 
 // Items are handed out dynamically (the transposed lists differ in length:
 // 36-153 query blocks per key block at the 2048 canvas, so a static
-// round-robin leaves the busiest CTA ~5% above the mean), still in head-major
-// order, so that the CTAs in flight share one head's Q, dO and dQ accumulator
-// in L2.  kItemConsumers: TMA lane 1, the row-vector producer, the MMA warp, 8 elementwise warps, 4
-// drain warps.
+// round-robin leaves the busiest CTA ~5% above the mean), in the order that
+// bwd_pre_kernel wrote.  kItemConsumers: TMA lane 1, the row-vector producer,
+// the MMA warp, 8 elementwise warps, 4 drain warps.
 constexpr int kItemSlots = 4, kItemConsumers = 15;
 
 template <int D>
