@@ -553,10 +553,6 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
             tmem_wait_st();
           }
         }
-        // all four 32-column loads in flight before one wait
-        uint32_t r[kBN];
-#pragma unroll
-        for (int g = 0; g < kBN / 32; ++g) tmem_ld32(s_col + g * 32, *reinterpret_cast<uint32_t(*)[32]>(&r[g * 32]));
         // the maximum that the previous tile used, from its warp (waited for on
         // an item's first tile too: it also says that the slot written below
         // was read)
@@ -568,8 +564,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
           if (t > 0) m_new = m_before = *const_cast<volatile float*>(&sm.m_row[(sc - 1) & 1][row]);
           return true;
         };
-        if (kAhead && !(ok = previous_max())) break;
-        tmem_wait_ld();
+        // all four 32-column loads in flight before one wait
+        uint32_t r[kBN];
+#pragma unroll
+        for (int g = 0; g < kBN / 32; ++g) tmem_ld32(s_col + g * 32, *reinterpret_cast<uint32_t(*)[32]>(&r[g * 32]));
+        if (kAhead) ok = previous_max();
+        tmem_wait_ld();  // also when that wait gave up: the loads must not land in registers or TMEM reused since
+        if (!ok) break;
         float s[kBN];
 #pragma unroll
         for (int x = 0; x < kBN; ++x) s[x] = __uint_as_float(r[x]);
