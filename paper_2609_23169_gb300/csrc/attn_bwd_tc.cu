@@ -205,9 +205,9 @@ UT_DEV void tmem_ld64(uint32_t taddr, uint32_t* r) {
 // row), off the elementwise warps' path; S and dP are computed once per pair.
 // A final kernel scales the accumulator by the softmax scale and writes dQ in
 // bf16.  Roles (512 threads, four warpgroups; the register file is rebalanced
-// with setmaxnreg): warpgroup 0 = warp 0 TMA, warp 1 TMEM owner + MMA issuer
-// and warp 2 lane 0 the row vectors; warpgroups 1-2 = 8 elementwise warps; warpgroup 3 = 4 dQ
-// drain warps.
+// with setmaxnreg): warpgroup 0 = warp 0 TMA of K, V and Q, warp 1 TMEM owner +
+// MMA issuer, warp 2 the row vectors and warp 3 TMA of dO (one lane each);
+// warpgroups 1-2 = 8 elementwise warps; warpgroup 3 = 4 dQ drain warps.
 // TMEM columns: R0 [0,128), RQ [128,256), dV [256,256+d), dK [384,384+d).
 // For d = 64 the A operand K^T of the dQ product is padded to 128 rows with a
 // zero sub-tile placed right after K, and the padding rows of RQ are ignored.
@@ -225,7 +225,7 @@ constexpr uint32_t kColR0 = 0, kColRQ = 128, kColFuDv = 256, kColFuDk = 384;
 // Items are handed out dynamically (the transposed lists differ in length:
 // 36-153 query blocks per key block at the 2048 canvas, so a static
 // round-robin leaves the busiest CTA ~5% above the mean), in the order that
-// bwd_pre_kernel wrote.  kItemConsumers: TMA lane 1, the row-vector producer,
+// bwd_pre_kernel wrote.  kItemConsumers: the dO and row-vector producers,
 // the MMA warp, 8 elementwise warps, 4 drain warps.
 constexpr int kItemSlots = 4, kItemConsumers = 15;
 
@@ -246,7 +246,7 @@ struct FusedSmem {
   uint64_t s_full, s_empty, dp_full, dp_empty, pt_full, pt_done, dst_full, ds_done, dq_empty;
   uint64_t acc_full, acc_empty, mma_done;
   uint64_t vec_full[2], vec_empty[2];
-  // the CTA's item sequence: TMA lane 0 takes the next item from the global
+  // the CTA's item sequence: warp 0 takes the next item from the global
   // counter and publishes it here; every other role reads the slots in order
   int32_t item[kItemSlots];
   uint64_t item_full[kItemSlots], item_empty[kItemSlots];
@@ -342,11 +342,13 @@ __global__ void __launch_bounds__(kFuThreads, 1)
   };
   if (wg == 0) {
     setmaxnreg_dec<kFuRegCtl>();
-    if (warp == 0) {
-      // lane 0: K, V of the item and the Q ring (Q is freed after dK += dS^T Q);
-      // lane 1: the dO ring (dO is freed after dV += P^T dO).
-      if (lane < 2) {
-        const bool is_q = lane == 0;
+    if (warp == 0 || warp == 3) {
+      // Warp 0: K, V of the item and the Q ring (Q is freed after dK += dS^T Q);
+      // warp 3: the dO ring (dO is freed after dV += P^T dO).  One lane each: two
+      // lanes of one warp wait for each other wherever the compiler lets them meet
+      // again (1024 canvas, d = 128: 1% of the launch).
+      if (lane == 0) {
+        const bool is_q = warp == 0;
         if (is_q) {
           tma_prefetch_desc(&tm_q);
           tma_prefetch_desc(&tm_k);
@@ -564,7 +566,6 @@ __global__ void __launch_bounds__(kFuThreads, 1)
     // into the swizzled tiles: lane l gives row l % 16 of 16, chunk g + l / 16.
     const uint32_t srow = quarter * 32 + (lane & 15), chunk_hi = lane >> 4;
     const uint32_t pt_row = smem_u32(sm.pt) + half * kChunk + srow * 128;
-    const uint32_t dst_row = smem_u32(sm.dst) + half * kChunk + srow * 128;
     const uint32_t vec_at = half * HC + (lane & 3) * 16;
     auto load_vec = [](const float* src, float (&v)[16]) {
 #pragma unroll
@@ -588,6 +589,19 @@ __global__ void __launch_bounds__(kFuThreads, 1)
       const int L = uniform(tl.count_warp());
       const int64_t gk = (int64_t)j * kTile + krow;
       const bool row_ok = gk < prm.N;
+      // Key rows past N are zeros, so S = 0 there and P = exp(0 - LSE) is infinite
+      // where LSE < -88.7: their rows of dS^T have to be zero, or dQ^T = K^T dS^T
+      // sums 0 * inf.  In the last key tile they are cleared once, and what the
+      // pairs compute for them goes over the same rows of P^T, which only reach
+      // rows of dV that are not written.  Nothing is added to the loop over the
+      // pairs but the choice of the row: selects on P or on dS^T, a test that is
+      // never true, a copy of the loop, the clearing by the MMA warp or products
+      // that leave those lanes out all cost more (1 to 14%; this -1 to 2%, and 4%
+      // with d = 64 and 64-row blocks on both sides).
+      const int key_rows = (int)min((int64_t)kTile, prm.N - (int64_t)j * kTile);
+      const uint32_t to_dst = smem_u32(sm.dst) - smem_u32(sm.pt);
+      const uint32_t ds_row[2] = {pt_row + ((int)srow < key_rows ? to_dst : 0),
+                                  pt_row + ((int)srow + 16 < key_rows ? to_dst : 0) + 2048};
       __nv_bfloat16* dv_row = prm.out0 + gk * prm.rs + (int64_t)h * D + half * HD;
       __nv_bfloat16* dk_row = prm.out1 + gk * prm.rs + (int64_t)h * D + half * HD;
       if (L <= 0) {
@@ -597,6 +611,11 @@ __global__ void __launch_bounds__(kFuThreads, 1)
             *reinterpret_cast<uint4*>(dk_row + e) = make_uint4(0, 0, 0, 0);
           }
         continue;
+      }
+      if (key_rows < (int)quarter * 32 + 32) {  // (the tile is free: the item before has been written out)
+        for (int x = max(key_rows - (int)quarter * 32, 0) * 8 + (int)lane; x < 32 * 8; x += 32)
+          *reinterpret_cast<uint4*>(sm.dst + half * kChunk + quarter * (32 * 128) + x * 16) = make_uint4(0, 0, 0, 0);
+        __syncwarp();
       }
       for (int t = 0; t < L; ++t) {
         const uint32_t qd = qd0 + t;
@@ -679,7 +698,7 @@ __global__ void __launch_bounds__(kFuThreads, 1)
           if (u == 0 && !(ok = warp_wait(&sm.ds_done, (qd & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns))) break;
 #pragma unroll
           for (int g = 0; g < 8; g += 2)
-            stmatrix_x4(dst_row + u * 2048 + (((g + chunk_hi) ^ (srow & 7)) << 4), dsk[2 * g], dsk[2 * g + 1],
+            stmatrix_x4(ds_row[u] + (((g + chunk_hi) ^ (srow & 7)) << 4), dsk[2 * g], dsk[2 * g + 1],
                         dsk[2 * g + 2], dsk[2 * g + 3]);
         }
         if (!ok) break;
