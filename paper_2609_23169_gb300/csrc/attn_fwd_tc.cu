@@ -686,8 +686,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
         // epilogue: O / l -> bf16, LSE (natural log)
         if (!(ok = warp_wait(&sm.l_full[is][quarter], (it >> 1) & 1, abort_flag, prm.status, prm.timeout_ns))) break;
         const float l_o = *const_cast<volatile float*>(&sm.l_row[is][row]);
-        // it is under the maximum that the last tile but one used, <= m
-        if (l_o > 0.f) l += l_o * ex2_approx(m_before - m);
+        // it is under the maximum that the last tile but one used, <= m (0 where
+        // there was none; a NaN has to come through)
+        if (l_o != 0.f) l += l_o * ex2_approx(m_before - m);
         if (!(ok = warp_wait(&sm.pv_done[last & 1], (last >> 1) & 1, abort_flag, prm.status, prm.timeout_ns))) break;
         tc_fence_after();
         uint32_t o[D];
