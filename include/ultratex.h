@@ -300,6 +300,10 @@ ut_status ut_block_mask(const ut_attn_shape* shape, int32_t mode,
  * for every head and query block i, S_i the list row_ptr/col_idx gives
  * (query blocks of b_q rows, listed key blocks of b_kv rows).
  * A query row whose block lists no key block gets O = 0 and LSE = -inf.
+ * A list holds a block at most once.  Its order is free, except for bf16 with
+ * b_q = 64, where two lists are merged and have to ascend (as ut_block_mask
+ * writes them); in the gradient that holds for the transposed lists with
+ * b_kv = 64.
  *   q, k, v, o  [N, H, d] token-major with shape->row_stride (dtype of shape).
  *   lse         [H, N] fp32 natural-log row normalisers (m + log sum exp).
  *   softmax_scale  1/sqrt(d) in the paper; any positive value accepted.

@@ -7,10 +7,10 @@
 // items form one stream; tile n of the stream belongs to softmax warpgroup
 // n & 1 and to S buffer n & 1.  Roles (384 threads, three warpgroups, registers
 // rebalanced with setmaxnreg):
-//   warp 0      TMA producers: lane 0 streams the items' Q tiles and the K tiles,
-//               lane 1 the V tiles, K and V each into a 3-stage ring of
-//               128B-swizzled shared tiles.  A K stage is released by the MMA
-//               that consumed it (S = Q K^T), a V stage by O += P V.
+//   warps 0, 2  TMA producers, one lane each: warp 0 streams the items' Q tiles
+//               and the K tiles, warp 2 the V tiles, K and V each into a 3-stage
+//               ring of 128B-swizzled shared tiles.  A K stage is released by
+//               the MMA that consumed it (S = Q K^T), a V stage by O += P V.
 //   warp 1      TMEM owner and MMA issuer: O += P_u V_u (P from TMEM, V from
 //               shared memory), then S_{u+2} = Q K_{u+2}^T (Q from TMEM, K from
 //               shared memory) into the buffer P_u was just read from.
@@ -67,6 +67,7 @@ constexpr int kFwdThreads = 384;
 constexpr int kFwdRegLaunch = 168, kFwdRegCtl = 88, kFwdRegSm = 208;
 static_assert(kFwdRegCtl + 2 * kFwdRegSm == 3 * kFwdRegLaunch, "setmaxnreg split must match the launch");
 constexpr int kStages = 3;                       // K and V ring depth
+constexpr int kRowSlots = 8;
 constexpr uint32_t kTileChunkBytes = 128 * 128;  // 128 rows x 128 bytes (64 bf16)
 constexpr uint32_t kColO = 256, kColQ = 384;     // TMEM column bases (Q: two buffers of 64 columns)
 
@@ -110,6 +111,11 @@ struct FwdSmem {
   uint64_t o_empty, mma_done;
   uint64_t m_full[2][4];       // [tile & 1][lane quarter]: row maxima published
   uint64_t l_full[2][4];       // [item & 1][lane quarter]: the other warpgroup's normalisers
+  // existing rows of the key tiles, by tile % kRowSlots (128-row blocks).  The K
+  // producer is at most three tiles ahead of S and S two ahead of P V, whose P
+  // needs the row maxima of every tile before it: a slot is read long before
+  // it is written again.
+  int32_t k_rows[kRowSlots];
   int32_t mine[kSortRounds];   // this CTA's items, where they are sorted
   float m_row[2][kBM];         // row maximum used by tile (tile & 1)
   float l_row[2][kBM];         // normaliser handed over, per item & 1
@@ -296,13 +302,17 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
 
   if (warp < 4) {
   setmaxnreg_dec<kFwdRegCtl>();
-  if (warp == 0) {
-    // ------------------------------------------------------------ producer
-    // lane 0 streams Q and K, lane 1 streams V: each ring is released by the
-    // MMA that consumes it (K after S = Q K^T, V after O += P V), so neither
-    // waits for the other.
-    if (lane < 2) {
-      const bool is_k = lane == 0;
+  if (warp == 0 || warp == 2) {
+    // ----------------------------------------------------------- producers
+    // Warp 0 streams Q and K, warp 2 streams V, one lane each: each ring is
+    // released by the MMA that consumes it (K after S = Q K^T, V after O += P V),
+    // so neither waits for the other.  As two lanes of one warp they did, wherever
+    // the compiler let the lanes meet again: 7,780 tokens, 24 heads, lists of 20%
+    // 139.6 -> 129.8 us, 512 canvas with d = 64 117 -> 111, 64-row blocks 2,360 ->
+    // 2,234 (85,202 tokens, 4 heads); a branch on the lane in the loop made it
+    // 20% slower.
+    if (lane == 0) {
+      const bool is_k = warp == 0;
       if (is_k) {
         tma_prefetch_desc(&tm_q);
         tma_prefetch_desc(&tm_k);
@@ -319,6 +329,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       const void* tmap = is_k ? static_cast<const void*>(&tm_k) : static_cast<const void*>(&tm_v);
       const void* tmap64 = is_k ? static_cast<const void*>(&tm_k64) : static_cast<const void*>(&tm_v64);
       uint32_t qi = 0, kv = 0;
+      const int cut_block = prm.N % kBN ? prm.nq - 1 : -1;
       bool ok = true;
       int k;
       for (int w = first_item(k); w < prm.n_items && ok; w = next_item(w, k)) {
@@ -335,9 +346,22 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
         }
         int j, jh;
         uint32_t bits;
+        bool held = false;  // 128-row blocks: the block that N cuts off, met before the end of the list
         for (; tl.next(j, jh, bits); ++kv) {
           const uint32_t st = kv % kStages, n = kv / kStages;
+          if (kMode == 0) {
+            // lists in any order: that block changes places with the last one, so
+            // that the softmax warps mask columns in an item's last tile only
+            const bool last = tl.tl.pa == tl.tl.na;
+            if (last && held) j = cut_block;
+            else if (!last && j == cut_block) {
+              held = true;
+              j = tl.tl.a[tl.tl.na - 1];
+            }
+          }
           if (!(ok = mbar_wait(&empty[st], (n & 1) ^ 1, abort_flag, prm.status, prm.timeout_ns))) break;
+          if (kMode == 0 && is_k)
+            *const_cast<volatile int*>(&sm.k_rows[kv % kRowSlots]) = j == cut_block ? (int)(prm.N % kBN) : kBN;
           mbar_expect_tx(&full[st], FwdSmem<D>::kKVBytes);
           uint8_t* dst = ring + st * FwdSmem<D>::kKVBytes;
           if (tl.pair) {  // two 64-row boxes: rows 0-63 and 64-127 of each 128-row sub-tile
@@ -352,7 +376,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
           }
         }
       }
-      // Drain: every copy this lane issued has landed before the CTA may exit.
+      // Drain: every copy this thread issued has landed before the CTA may exit.
       auto drain = [&](uint64_t* bar, uint32_t parity) {
         if (!mbar_drain(bar, parity, kDrainTimeoutNs)) set_status(prm.status, UT_ERR_TIMEOUT);
       };
@@ -524,11 +548,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
       }
       const uint32_t t0 = (sc0 ^ wgi) & 1;  // this warpgroup's first tile of the item
       if (t0 == 0 && !(ok = load_q())) break;
-      // lists ascend: with 128-row blocks only the last tile can be ragged
       int j = 0, jh = -1;
       uint32_t bits = 15u;
-      if (kMode == 0) j = tl.tl.a[L - 1];
-      else if (t0) tl.next(j, jh, bits);
+      if (kMode != 0 && t0) tl.next(j, jh, bits);
       float m_before = 0.f;  // the maximum the previous tile of the stream used
       float m = 0.f, l = 0.f;  // row maximum in use and this warpgroup's part of the normaliser under it
       for (int t = t0; t < L; t += 2) {
@@ -545,8 +567,13 @@ __global__ void __launch_bounds__(kFwdThreads, 1)
         // or not, sit in the middle of every tile's instruction stream.
         if (kMode != 0 || t == L - 1) {
           const int e0 = tl.pair ? 64 : kBN;  // columns that belong to the low (or only) listed block
-          const int64_t nv0 = prm.N - (tl.pair ? 64 * (int64_t)PairList::load_lo(j, jh) : (int64_t)j * kBN);
-          const int64_t nv1 = tl.pair ? prm.N - 64 * (int64_t)PairList::load_hi(j, jh) : 64;
+          int64_t nv0, nv1 = 64;
+          if constexpr (kMode == 0) {
+            nv0 = *const_cast<volatile int*>(&sm.k_rows[sc % kRowSlots]);
+          } else {
+            nv0 = prm.N - (tl.pair ? 64 * (int64_t)PairList::load_lo(j, jh) : (int64_t)j * kBN);
+            nv1 = tl.pair ? prm.N - 64 * (int64_t)PairList::load_hi(j, jh) : 64;
+          }
           if (__builtin_expect(nv0 < e0 || nv1 < 64, 0)) {
             for (int x = (int)nv0; x < e0; ++x) tmem_st1(s_col + x, 0xff800000u);
             for (int x = (int)nv1; x < 64; ++x) tmem_st1(s_col + 64 + x, 0xff800000u);
