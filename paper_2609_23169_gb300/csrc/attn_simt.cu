@@ -417,7 +417,9 @@ UT_DEV void f32_tile(const F32Args& a, F32Smem<D, MODE>& sm, int part) {
   add(ex1);
   float f[4];
 #pragma unroll
-  for (int y = 0; y < 4; ++y) f[y] = MODE == kFwd ? (l[y] > 0.f ? 1.f / l[y] : 0.f) : 1.f;
+  // a row that lists nothing gets O = 0; one whose scores are all -inf has no
+  // softmax (0 / 0)
+  for (int y = 0; y < 4; ++y) f[y] = MODE == kFwd ? (l[y] > 0.f ? 1.f / l[y] : (pieces > 0 ? NAN : 0.f)) : 1.f;
   store_rows<D, kVec>(a.out0, r0, valid, off, a.rs, rg, c, acc, f);
   if constexpr (MODE == kDkv) store_rows<D, kVec>(a.out1, r0, valid, off, a.rs, rg, c, acc2, f);
   if (MODE == kFwd && c == 0) {
