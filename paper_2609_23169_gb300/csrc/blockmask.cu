@@ -25,7 +25,6 @@ constexpr int kPoolThreads = 128;
 constexpr int kSelThreads = 128;
 constexpr int kSelCols = 256;      // key blocks per tile of scores
 constexpr int kSelRows = 16;       // query blocks per CTA (fewer when N_k is large)
-constexpr int kSelRegKeys = 32;    // keys a lane holds in registers: N_k <= 1024
 
 template <typename T>
 struct Vec8;
@@ -176,6 +175,54 @@ UT_DEV void select_row(const float* srow, int nk, int k, int lane, uint32_t& thr
       k, lo, hi, nk, thr, equal);
 }
 
+// The same for rows that do not fit registers (N_k > 2048), where each of the
+// search's passes would read the row from shared memory again: four passes by 8
+// bits, counts of the warp in hw[256] (shared).  6,656 key blocks, 1 head: 3,700
+// -> 2,530 us for the lists (the search 12 passes; these four were there before it
+// and took 3,630 with the scores of that time); 1,332 key blocks, 24 heads of d =
+// 64, 48 keys a lane in registers: 1,080 -> 848 (898 with these passes and the
+// scores of that time).
+UT_DEV void select_row_radix(const float* srow, int nk, int k, int lane, uint32_t* hw, uint32_t& thr, int& equal) {
+  uint32_t prefix = 0, pmask = 0;
+  for (int shift = 24; shift >= 0; shift -= 8) {
+    for (int b = lane; b < 256; b += 32) hw[b] = 0;
+    __syncwarp();
+    for (int j = lane; j < nk; j += 32) {
+      const uint32_t u = order_key(srow[j]);
+      if ((u & pmask) == prefix) atomicAdd(&hw[(u >> shift) & 255u], 1u);
+    }
+    __syncwarp();
+    // lane l owns bins 255 - 8 l .. 248 - 8 l; one lane finds the bin that holds rank k
+    uint32_t cnt[8], local = 0;
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+      cnt[x] = hw[255 - 8 * lane - x];
+      local += cnt[x];
+    }
+    uint32_t incl = local;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    uint32_t digit = 255 - 8 * lane, above = incl - local;
+    const bool here = above < (uint32_t)k && (uint32_t)k <= incl;
+#pragma unroll
+    for (int x = 0; x < 7; ++x) {
+      if (above + cnt[x] >= (uint32_t)k) break;
+      above += cnt[x];
+      --digit;
+    }
+    const int src = __ffs(__ballot_sync(0xffffffffu, here)) - 1;
+    digit = __shfl_sync(0xffffffffu, digit, src);
+    k -= (int)__shfl_sync(0xffffffffu, above, src);
+    prefix |= digit << shift;
+    pmask |= 0xFFu << shift;
+    __syncwarp();
+  }
+  thr = prefix;
+  equal = k;
+}
+
 // grid (H, ceil(nq / R)); dynamic smem: pooled query rows [d][kRows], a slice of
 // pooled keys [kE][kSelCols], scores [R][nk].  Rows are query blocks (nq per
 // head), columns key blocks (nk).
@@ -185,10 +232,13 @@ UT_DEV void select_row(const float* srow, int nk, int k, int lane, uint32_t& thr
 // us at the 2048 canvas; 8 rows x 4 key blocks read 48 for 32 (and with the
 // search above instead of 32 passes by bits 263 -> 194; 282 with the keys read
 // from global memory and a radix select over shared counters).  Slices are
-// staged d-major, 4-column groups exchanged by (d / 4) % 8 so that neither the
-// transposing stores nor the reads conflict.  A sum runs over d in order, as
-// one FMA chain.
-template <int kRows, int kE>  // rows a tile holds, d per staged slice of pool(K)
+// staged d-major, 4-column groups exchanged by their d / 4 in the slice so that
+// neither the transposing stores nor the reads conflict.  A sum runs over d in
+// order, as one FMA chain.
+// kRows: rows a tile holds; kE: d per staged slice of pool(K); kLong: N_k > 1024 (a
+// kernel of its own: the selections of long rows would lengthen the code that a
+// small call has to fetch, 11.5 -> 12.6 us at 100 tokens)
+template <int kRows, int kE, bool kLong>
 __global__ void __launch_bounds__(kSelThreads) score_select_kernel(const float* __restrict__ pooled, int H, int d,
                                                                    int nq, int nk, int R, int k_rho,
                                                                    int32_t* __restrict__ row_ptr,
@@ -267,36 +317,29 @@ __global__ void __launch_bounds__(kSelThreads) score_select_kernel(const float* 
     }
   }
   __syncthreads();
+  static_assert(kE * kSelCols >= kSelThreads / 32 * 256, "256 counts a warp must fit over the last slice");
   const int lane = tid & 31, w = tid >> 5, W = (nk + 31) / 32;
   const uint32_t lt_mask = (1u << lane) - 1u;
   for (int r = w; r < rows; r += kSelThreads / 32) {
     const float* srow = sc + r * nk;
     uint32_t thr = 0;
     int equal = 0;
-    if (W <= 8) {
+    if constexpr (kLong) {
+      if (W <= 48) {
+        select_row<48>(srow, nk, k_rho, lane, thr, equal);
+      } else if (W <= 64) {
+        select_row<64>(srow, nk, k_rho, lane, thr, equal);
+      } else {
+        select_row_radix(srow, nk, k_rho, lane, reinterpret_cast<uint32_t*>(kt) + w * 256, thr, equal);
+      }
+    } else if (W <= 8) {
       select_row<8>(srow, nk, k_rho, lane, thr, equal);
     } else if (W <= 16) {
       select_row<16>(srow, nk, k_rho, lane, thr, equal);
     } else if (W <= 24) {
       select_row<24>(srow, nk, k_rho, lane, thr, equal);
-    } else if (W <= kSelRegKeys) {
-      select_row<kSelRegKeys>(srow, nk, k_rho, lane, thr, equal);
     } else {
-      uint32_t lo = 0xffffffffu, hi = 0u;
-      for (int j = lane; j < nk; j += 32) {
-        const uint32_t u = order_key(srow[j]);
-        lo = min(lo, u);
-        hi = max(hi, u);
-      }
-      lo = __reduce_min_sync(0xffffffffu, lo);
-      hi = __reduce_max_sync(0xffffffffu, hi);
-      select_kth(
-          [&](uint32_t cand) {
-            int n = 0;
-            for (int j = lane; j < nk; j += 32) n += order_key(srow[j]) >= cand;
-            return n;
-          },
-          k_rho, lo, hi, nk, thr, equal);
+      select_row<32>(srow, nk, k_rho, lane, thr, equal);
     }
     // all keys above thr, and the first `equal` ones at it
     const int row = h * nq + i0 + r;
@@ -475,14 +518,14 @@ __global__ void bitmap_fill_kernel(const uint8_t* __restrict__ bm, int H, int nq
 }
 
 // ----------------------------------------------------------------- launchers
-template <int kRows, int kE>
+template <int kRows, int kE, bool kLong>
 static cudaError_t launch_score_select(const float* pooled, int H, int d, int nq, int nk, int R, int k_rho,
                                        int32_t* row_ptr, int32_t* col_idx, uint32_t* bits, cudaStream_t stream) {
   const size_t smem = ((size_t)kRows * d + (size_t)kE * kSelCols + (size_t)R * nk) * sizeof(float);
   cudaError_t e =
-      cudaFuncSetAttribute(score_select_kernel<kRows, kE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(score_select_kernel<kRows, kE, kLong>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  score_select_kernel<kRows, kE><<<dim3(H, (nq + R - 1) / R), kSelThreads, smem, stream>>>(
+  score_select_kernel<kRows, kE, kLong><<<dim3(H, (nq + R - 1) / R), kSelThreads, smem, stream>>>(
       pooled, H, d, nq, nk, R, k_rho, row_ptr, col_idx, bits);
   return cudaGetLastError();
 }
@@ -522,9 +565,11 @@ cudaError_t launch_block_mask_topk(const MaskProblem& p, const void* q, const vo
   int R = (64 * 1024) / (nk * 4);
   R = R < 1 ? 1 : (R > kSelRows ? kSelRows : R);
   const bool roomy = ((size_t)4 * d + 16 * kSelCols + (size_t)R * nk) * sizeof(float) <= 232448;  // 227 KB a block
-  auto launch = R > 8 ? launch_score_select<16, 16>
-                      : (R > 4 ? launch_score_select<8, 16>
-                               : (roomy ? launch_score_select<4, 16> : launch_score_select<4, 4>));
+  auto launch = nk <= 1024 ? launch_score_select<16, 16, false>
+                : R > 8    ? launch_score_select<16, 16, true>
+                : R > 4    ? launch_score_select<8, 16, true>
+                : roomy    ? launch_score_select<4, 16, true>
+                           : launch_score_select<4, 4, true>;
   const cudaError_t e = launch(pooled, H, d, nq, nk, R, k_rho, row_ptr, col_idx, bits, stream);
   if (e != cudaSuccess) return e;
   if (col_ptr_t && row_idx_t)
