@@ -367,13 +367,18 @@ __global__ void __launch_bounds__(kSelThreads) score_select_kernel(const float* 
 
 // grid (H, ceil(nk / 32)): the lists of 32 key blocks of one head from the bit
 // mask [H, nq, W].  Every row holds k_rho entries, so a head's entries start at
-// h * nq * k_rho, and what lies before these 32 columns is a population count
-// over the words to their left: no pass over all counts, no second launch
-// (count, scan and fill took 67 us at the 2048 canvas, this launch about 20).  A warp owns a run of
-// 32-row groups; ballots turn 32 rows x 32 columns round, lane c then holding
-// column c's rows.
+// h * nq * k_rho, and what lies before these 32 columns is found here: no pass
+// over all counts, no second launch (count, scan and fill took 67 us at the 2048
+// canvas, this launch about 20).  Up to kTransWords words to the left it is a
+// population count over them; further right, where those words would be read
+// again and again (the cube of the number of blocks), a binary search in each
+// row's list (666 key blocks: the lists take 62.6 us counted, 65.2 searched; 2,048:
+// 751 and 637; 6,656: 2,719 and 2,525).  A warp owns a run of 32-row groups;
+// ballots turn 32 rows x 32 columns round, lane c then holding column c's rows.
 constexpr int kTransThreads = 256;
-__global__ void __launch_bounds__(kTransThreads) transpose_kernel(const uint32_t* __restrict__ bits, int H, int nq,
+constexpr int kTransWords = 32;  // words to the left that are counted
+__global__ void __launch_bounds__(kTransThreads) transpose_kernel(const uint32_t* __restrict__ bits,
+                                                                  const int32_t* __restrict__ col_idx, int H, int nq,
                                                                   int nk, int k_rho, int32_t* __restrict__ col_ptr,
                                                                   int32_t* __restrict__ row_idx) {
   constexpr int kWarps = kTransThreads / 32;
@@ -382,8 +387,21 @@ __global__ void __launch_bounds__(kTransThreads) transpose_kernel(const uint32_t
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t* hb = bits + (int64_t)h * nq * W;
   int before = 0;
-  for (int i = threadIdx.x; i < nq; i += kTransThreads)
-    for (int x = 0; x < wc; ++x) before += __popc(hb[(int64_t)i * W + x]);
+  if (wc <= kTransWords) {
+    for (int i = threadIdx.x; i < nq; i += kTransThreads)
+      for (int x = 0; x < wc; ++x) before += __popc(hb[(int64_t)i * W + x]);
+  } else {
+    for (int i = threadIdx.x; i < nq; i += kTransThreads) {
+      const int32_t* list = col_idx + ((int64_t)h * nq + i) * k_rho;
+      int lo = 0, hi = k_rho;  // entries below column 32 wc
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (list[mid] < 32 * wc) lo = mid + 1;
+        else hi = mid;
+      }
+      before += lo;
+    }
+  }
   before = __reduce_add_sync(0xffffffffu, before);
   const int groups = (nq + 31) / 32, per = (groups + kWarps - 1) / kWarps;
   const int g0 = min(groups, w * per), g1 = min(groups, g0 + per);
@@ -573,8 +591,8 @@ cudaError_t launch_block_mask_topk(const MaskProblem& p, const void* q, const vo
   const cudaError_t e = launch(pooled, H, d, nq, nk, R, k_rho, row_ptr, col_idx, bits, stream);
   if (e != cudaSuccess) return e;
   if (col_ptr_t && row_idx_t)
-    transpose_kernel<<<dim3(H, (nk + 31) / 32), kTransThreads, 0, stream>>>(bits, H, nq, nk, k_rho, col_ptr_t,
-                                                                          row_idx_t);
+    transpose_kernel<<<dim3(H, (nk + 31) / 32), kTransThreads, 0, stream>>>(bits, col_idx, H, nq, nk, k_rho,
+                                                                          col_ptr_t, row_idx_t);
   return cudaGetLastError();
 }
 
