@@ -448,41 +448,47 @@ __global__ void __launch_bounds__(kTransThreads) transpose_kernel(const uint32_t
   }
 }
 
-// One side of the bitmap's lists: rows, or columns for the transpose.
-struct ListSide {
-  int32_t* ptr;   // [lines + 1]
-  int32_t* idx;
-};
+// Line l = (h, a): a row i of [H][nq][nk], or a column j for the transpose; one
+// warp per line.  Rows and columns are functions of their own so that a line's
+// loads can run ahead of its stores (one function over either side's pointers, and
+// the scan's counts read one by one: 47.8 us for the rows' lists of the 2048
+// canvas against 33.3, 80.4 against 66.4 with the transpose).
+template <bool kCols>
+UT_DEV uint8_t bitmap_at(const uint8_t* __restrict__ bm, int h, int nq, int nk, int a, int b) {
+  return kCols ? bm[((int64_t)h * nq + b) * nk + a] : bm[((int64_t)h * nq + a) * nk + b];
+}
 
-// One warp per line.  Line l = (h, a): a row i of [H][nq][nk] (blockIdx.y = 0) or
-// a column j (blockIdx.y = 1).
-__global__ void bitmap_count_kernel(const uint8_t* __restrict__ bm, int H, int nq, int nk, ListSide rows,
-                                    ListSide cols) {
-  const bool transposed = blockIdx.y == 1;
-  const int n_lines = transposed ? nk : nq;
+template <bool kCols>
+UT_DEV void count_line(const uint8_t* __restrict__ bm, int H, int nq, int nk, int32_t* __restrict__ counts) {
+  const int n_lines = kCols ? nk : nq, len = kCols ? nq : nk;
   const int line = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (line >= H * n_lines) return;
   const int h = line / n_lines, a = line % n_lines;
-  const int len = transposed ? nq : nk;
   const int lane = threadIdx.x & 31;
   int c = 0;
-  for (int b = lane; b < len; b += 32) {
-    uint8_t v = transposed ? bm[((int64_t)h * nq + b) * nk + a] : bm[((int64_t)h * nq + a) * nk + b];
-    c += v != 0;
-  }
+  for (int b = lane; b < len; b += 32) c += bitmap_at<kCols>(bm, h, nq, nk, a, b) != 0;
   for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) (transposed ? cols : rows).ptr[line] = c;
+  if (lane == 0) counts[line] = c;
+}
+
+// blockIdx.y: 0 the rows, 1 the columns
+__global__ void bitmap_count_kernel(const uint8_t* __restrict__ bm, int H, int nq, int nk,
+                                    int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_ptr) {
+  if (blockIdx.y == 0) count_line<false>(bm, H, nq, nk, row_ptr);
+  else count_line<true>(bm, H, nq, nk, col_ptr);
 }
 
 // Exclusive scan in place of the counts ptr[0..n) into ptr[0..n], one CTA a side.
-__global__ void __launch_bounds__(1024) scan_kernel(int n_rows, int n_cols, ListSide rows, ListSide cols) {
+__global__ void __launch_bounds__(1024) scan_kernel(int n_rows, int n_cols, int32_t* row_ptr, int32_t* col_ptr) {
   __shared__ int64_t warp_tot[32];
   const int n = blockIdx.x ? n_cols : n_rows;
-  int32_t* ptr = (blockIdx.x ? cols : rows).ptr;
+  int32_t* ptr = blockIdx.x ? col_ptr : row_ptr;
   const int tid = threadIdx.x;
   const int per = (n + 1023) / 1024;
   const int a = min(n, tid * per), b = min(n, a + per);
+  constexpr int kAhead = 8;  // counts loaded before any is replaced by its prefix
   int64_t local = 0;
+#pragma unroll kAhead
   for (int t = a; t < b; ++t) local += ptr[t];
   int64_t incl = local;
   const int lane = tid & 31, w = tid >> 5;
@@ -495,35 +501,33 @@ __global__ void __launch_bounds__(1024) scan_kernel(int n_rows, int n_cols, List
   int64_t wpre = 0;
   for (int i = 0; i < w; ++i) wpre += warp_tot[i];
   int64_t run = wpre + incl - local;
-  for (int t = a; t < b; ++t) {
-    const int c = ptr[t];
-    ptr[t] = (int32_t)run;
-    run += c;
+  for (int t = a; t < b; t += kAhead) {
+    int c[kAhead];
+#pragma unroll
+    for (int x = 0; x < kAhead; ++x) c[x] = t + x < b ? ptr[t + x] : 0;
+#pragma unroll
+    for (int x = 0; x < kAhead; ++x) {
+      if (t + x < b) ptr[t + x] = (int32_t)run;
+      run += c[x];
+    }
   }
   if (tid == 1023) ptr[n] = (int32_t)(wpre + incl);
 }
 
-__global__ void bitmap_fill_kernel(const uint8_t* __restrict__ bm, int H, int nq, int nk, ListSide rows,
-                                   ListSide cols, int64_t cap, int32_t* status) {
-  const bool transposed = blockIdx.y == 1;
-  const int32_t* ptr = (transposed ? cols : rows).ptr;
-  int32_t* out = (transposed ? cols : rows).idx;
-  const int n_lines = transposed ? nk : nq;
+template <bool kCols>
+UT_DEV void fill_line(const uint8_t* __restrict__ bm, int H, int nq, int nk, const int32_t* __restrict__ ptr,
+                      int32_t* __restrict__ out, int64_t cap, int32_t* status) {
+  const int n_lines = kCols ? nk : nq, len = kCols ? nq : nk;
   const int line = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (line >= H * n_lines) return;
   const int h = line / n_lines, a = line % n_lines;
-  const int len = transposed ? nq : nk;
   const int lane = threadIdx.x & 31;
   const uint32_t lt_mask = (1u << lane) - 1u;
   int64_t pos = ptr[line];
   bool overflow = false;
   for (int b0 = 0; b0 < len; b0 += 32) {
     const int b = b0 + lane;
-    bool on = false;
-    if (b < len) {
-      uint8_t v = transposed ? bm[((int64_t)h * nq + b) * nk + a] : bm[((int64_t)h * nq + a) * nk + b];
-      on = v != 0;
-    }
+    const bool on = b < len && bitmap_at<kCols>(bm, h, nq, nk, a, b) != 0;
     const uint32_t bal = __ballot_sync(0xffffffffu, on);
     if (on) {
       int64_t p = pos + __popc(bal & lt_mask);
@@ -533,6 +537,14 @@ __global__ void bitmap_fill_kernel(const uint8_t* __restrict__ bm, int H, int nq
     pos += __popc(bal);
   }
   if (__any_sync(0xffffffffu, overflow) && lane == 0) set_status(status, UT_ERR_CAPACITY);
+}
+
+__global__ void bitmap_fill_kernel(const uint8_t* __restrict__ bm, int H, int nq, int nk,
+                                   const int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx,
+                                   const int32_t* __restrict__ col_ptr, int32_t* __restrict__ row_idx, int64_t cap,
+                                   int32_t* status) {
+  if (blockIdx.y == 0) fill_line<false>(bm, H, nq, nk, row_ptr, col_idx, cap, status);
+  else fill_line<true>(bm, H, nq, nk, col_ptr, row_idx, cap, status);
 }
 
 // ----------------------------------------------------------------- launchers
@@ -600,13 +612,13 @@ cudaError_t launch_block_mask_bitmap(const MaskProblem& p, const uint8_t* bitmap
                                      int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap, int32_t* status,
                                      cudaStream_t stream) {
   const bool with_cols = col_ptr_t && row_idx_t;
-  const ListSide rows{row_ptr, col_idx}, cols{col_ptr_t, row_idx_t};
   const int lines = p.H * (with_cols && p.nk > p.nq ? p.nk : p.nq);
   const dim3 grid((lines + 7) / 8, with_cols ? 2 : 1);
   if (lines == 0) return cudaSuccess;
-  bitmap_count_kernel<<<grid, 256, 0, stream>>>(bitmap, p.H, p.nq, p.nk, rows, cols);
-  scan_kernel<<<with_cols ? 2 : 1, 1024, 0, stream>>>(p.H * p.nq, p.H * p.nk, rows, cols);
-  bitmap_fill_kernel<<<grid, 256, 0, stream>>>(bitmap, p.H, p.nq, p.nk, rows, cols, col_cap, status);
+  bitmap_count_kernel<<<grid, 256, 0, stream>>>(bitmap, p.H, p.nq, p.nk, row_ptr, col_ptr_t);
+  scan_kernel<<<with_cols ? 2 : 1, 1024, 0, stream>>>(p.H * p.nq, p.H * p.nk, row_ptr, col_ptr_t);
+  bitmap_fill_kernel<<<grid, 256, 0, stream>>>(bitmap, p.H, p.nq, p.nk, row_ptr, col_idx, col_ptr_t, row_idx_t, col_cap,
+                                              status);
   return cudaGetLastError();
 }
 
