@@ -24,7 +24,6 @@
 namespace ut {
 
 constexpr int kSamplerThreads = 256;
-constexpr int kBatch = 4;  // vectors a thread of the composite takes at once
 
 static int stream_grid(int64_t threads, int sms) {
   const int64_t need = (threads + kSamplerThreads - 1) / kSamplerThreads;
@@ -74,13 +73,19 @@ __global__ void __launch_bounds__(kSamplerThreads) fg_euler_kernel(const int32_t
   }
 }
 
-// Bound by the latency of its dependent loads (mask, then the tile's row) at 10
-// MB: a thread takes kBatch vectors at once, all masks, then all rows, then the
-// stores, and the index arithmetic is 32-bit where it fits (two 64-bit divisions
-// a vector cost more than its loads).  2048 target canvas, 64 bf16 channels: 6.1
-// -> 5.0 us.  (The same for the Euler update, whose one division was 32-bit
-// already, gave nothing: 5.9 against 6.3.)
-template <typename I>
+// Small canvases are bound by the latency of the dependent loads (mask, then the
+// tile's row), large ones by HBM; the index arithmetic is 32-bit where it fits
+// (two 64-bit divisions a vector cost more than its loads).  A thread takes
+// kBatch vectors at once, all masks, then all rows, then the stores: 4 where
+// that makes the whole canvas one batch of the grid (2048 target canvas, 64 bf16
+// channels, 0.8 M vectors: 4.1 us against 4.4 with one, 5.0 with 64-bit indices),
+// one elsewhere: fewer vectors than threads only lengthen the chain (1,000 rows
+// of 64 channels: 1.7 us against 2.3 with four), and over several batches the
+// four streams apart cost more than they hide (53,248 rows of 512 channels: 11.1
+// against 11.4, 212,992 of 3,072: 220 against 262; 238 with 64-bit indices).
+// (The same for the Euler update, whose one division was 32-bit already, gave
+// nothing: 5.9 against 6.3.)
+template <typename I, int kBatch>
 __global__ void __launch_bounds__(kSamplerThreads) fg_composite_kernel(const uint8_t* __restrict__ mask, int64_t T,
                                                                        uint8_t* __restrict__ z,
                                                                        const uint8_t* __restrict__ tile,
@@ -137,16 +142,17 @@ cudaError_t launch_fg_composite(const uint8_t* mask, int64_t T, void* z, const v
                                 int64_t row_bytes, int sms, cudaStream_t stream) {
   if (T == 0) return cudaSuccess;
   const int64_t vectors = T * (row_bytes >> 4);
-  const int grid = stream_grid((vectors + kBatch - 1) / kBatch, sms);
-  uint8_t* zb = static_cast<uint8_t*>(z);
-  const uint8_t* tb = static_cast<const uint8_t*>(tile);
+  const int64_t most = (int64_t)sms * 8 * kSamplerThreads;  // threads of the largest grid
+  const int batch = vectors > most && vectors <= 4 * most ? 4 : 1;
+  const int grid = stream_grid((vectors + batch - 1) / batch, sms);
   // the indices that the loop forms stay below the vectors plus two batches of
   // the whole grid
-  const bool small = vectors + 2 * (int64_t)grid * kSamplerThreads * kBatch < ((int64_t)1 << 31);
-  if (small && period < ((int64_t)1 << 31))
-    fg_composite_kernel<int32_t><<<grid, kSamplerThreads, 0, stream>>>(mask, T, zb, tb, period, row_bytes);
-  else
-    fg_composite_kernel<int64_t><<<grid, kSamplerThreads, 0, stream>>>(mask, T, zb, tb, period, row_bytes);
+  const bool small = vectors + 2 * (int64_t)grid * kSamplerThreads * batch < ((int64_t)1 << 31) &&
+                     period < ((int64_t)1 << 31);
+  auto kernel = !small ? fg_composite_kernel<int64_t, 1>
+                       : (batch == 4 ? fg_composite_kernel<int32_t, 4> : fg_composite_kernel<int32_t, 1>);
+  kernel<<<grid, kSamplerThreads, 0, stream>>>(mask, T, static_cast<uint8_t*>(z), static_cast<const uint8_t*>(tile),
+                                               period, row_bytes);
   return cudaGetLastError();
 }
 
