@@ -306,8 +306,7 @@ ut_status ut_block_mask(const ut_attn_shape* shape, int32_t mode, const void* q,
     if (!q || !k || !aligned16(q) || !aligned16(k)) return UT_ERR_INVALID_ARG;
     const int32_t kr = ut_topk_count(rho, nk);
     if ((int64_t)shape->n_heads * nq * kr > col_cap || !col_idx) return UT_ERR_CAPACITY;
-    return from_cuda(launch_block_mask_topk(p, q, k, kr, row_ptr, col_idx, col_ptr_t, row_idx_t, col_cap, ws,
-                                            dev_status, device_sms(), s));
+    return from_cuda(launch_block_mask_topk(p, q, k, kr, row_ptr, col_idx, col_ptr_t, row_idx_t, ws, s));
   }
   if (!bitmap || !dev_status) return UT_ERR_INVALID_ARG;
   if (col_cap > 0 && !col_idx) return UT_ERR_INVALID_ARG;

@@ -560,6 +560,11 @@ static cudaError_t launch_score_select(const float* pooled, int H, int d, int nq
   return cudaGetLastError();
 }
 
+// More than the kernels use, and kept: a workspace of the size that was asked for
+// before is still enough, and one that was refused still is.  Top-K holds the
+// pooled rows and the bit mask, 4 ceil(nk / 32) bytes a row, which fits the nk
+// bytes a row counted here (for nk < 4 with the counts after them); the bitmap
+// mode counts into the pointer arrays and uses none.
 size_t block_mask_ws(const MaskProblem& p, int mode) {
   const size_t H = p.H, nq = p.nq, nk = p.nk, d = p.d;
   size_t counts = (H * (nq > nk ? nq : nk) + 1) * sizeof(int32_t);
@@ -570,13 +575,10 @@ size_t block_mask_ws(const MaskProblem& p, int mode) {
 }
 
 cudaError_t launch_block_mask_topk(const MaskProblem& p, const void* q, const void* k, int k_rho, int32_t* row_ptr,
-                                   int32_t* col_idx, int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap,
-                                   void* ws, int32_t* status, int sms, cudaStream_t stream) {
-  (void)sms;
+                                   int32_t* col_idx, int32_t* col_ptr_t, int32_t* row_idx_t, void* ws,
+                                   cudaStream_t stream) {
   const int H = p.H, nq = p.nq, nk = p.nk, d = p.d;
   float* pooled = static_cast<float*>(ws);
-  // bit mask: 4 ceil(nk / 32) bytes a row, within the bytes that block_mask_ws
-  // counts for the mask (nk a row) and, for nk < 4, the counts after it
   uint32_t* bits = reinterpret_cast<uint32_t*>(pooled + (size_t)H * (nq + nk) * d);
   const int elems = p.dtype == UT_BF16 ? 8 : 4;
   dim3 pg(nq > nk ? nq : nk, 2, (H * d / elems + kPoolThreads - 1) / kPoolThreads);

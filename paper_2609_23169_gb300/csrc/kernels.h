@@ -42,8 +42,8 @@ struct MaskProblem {
 };
 size_t block_mask_ws(const MaskProblem& p, int mode);
 cudaError_t launch_block_mask_topk(const MaskProblem& p, const void* q, const void* k, int k_rho, int32_t* row_ptr,
-                                   int32_t* col_idx, int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap,
-                                   void* ws, int32_t* status, int sms, cudaStream_t stream);
+                                   int32_t* col_idx, int32_t* col_ptr_t, int32_t* row_idx_t, void* ws,
+                                   cudaStream_t stream);
 cudaError_t launch_block_mask_bitmap(const MaskProblem& p, const uint8_t* bitmap, int32_t* row_ptr, int32_t* col_idx,
                                      int32_t* col_ptr_t, int32_t* row_idx_t, int64_t col_cap, int32_t* status,
                                      cudaStream_t stream);
