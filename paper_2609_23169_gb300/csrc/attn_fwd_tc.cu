@@ -40,7 +40,8 @@
 // Measured against one warpgroup, same clocks: 2048 canvas, Top-K 0.12, 7,545 ->
 // 7,384 us in a loop (6,972 -> 6,783 after a pause: in a loop the card is at its
 // 1.4 kW cap, and what the kernel gains in cycles the clock gives back, 1,815 ->
-// 1,732 MHz); d = 64 forward and backward at 512 418 -> 398 us.
+// 1,732 MHz); d = 64 forward and backward at 512 418 -> 398 us.  With the two
+// producers apart (below) 7,130 and 6,350 us at 2048, 203 -> 193 at 512.
 // Blocks of 64 rows (b_q or b_kv) are served by the same 128 x 128 tiles:
 //   b_kv = 64:  two listed 64-row key blocks fill one 128-row key tile (two
 //               TMA boxes per operand, PairList): consecutive entries of the
@@ -67,7 +68,7 @@ constexpr int kFwdThreads = 384;
 constexpr int kFwdRegLaunch = 168, kFwdRegCtl = 88, kFwdRegSm = 208;
 static_assert(kFwdRegCtl + 2 * kFwdRegSm == 3 * kFwdRegLaunch, "setmaxnreg split must match the launch");
 constexpr int kStages = 3;                       // K and V ring depth
-constexpr int kRowSlots = 8;
+constexpr int kRowSlots = 8;                     // key tiles whose row counts are kept
 constexpr uint32_t kTileChunkBytes = 128 * 128;  // 128 rows x 128 bytes (64 bf16)
 constexpr uint32_t kColO = 256, kColQ = 384;     // TMEM column bases (Q: two buffers of 64 columns)
 
@@ -78,10 +79,15 @@ constexpr uint32_t kColO = 256, kColQ = 384;     // TMEM column bases (Q: two bu
 // or order, so every CTA computes the same order for itself, in its still unused
 // K ring: items by length, longest first, equal ones by index, dealt out
 // boustrophedon (202 steps there).  Only where it pays: a few items per CTA
-// (the more there are the better index order evens out), K and V of all heads in
-// L2 at once (the order gives up that neighbours share a head: with 43 MB a head
-// an order across heads costs 31%), index order at least 5% off the mean, and
-// 128-row blocks on both sides.  512 canvas: 219 -> 207 us.
+// (the more there are the better index order evens out; the scratch holds 4,096
+// in all), index order at least 5% off the mean, 128-row blocks on both sides, and
+// K and V of all heads within 96 MiB, since the order gives up that neighbours
+// share a head in L2.  512 canvas: 219 -> 207 us when it
+// was made (193 now).  Sorted against index order, d = 128, 24 heads, lists of
+// 20%, K + V of 59 / 91 / 105 / 117 / 152 / 199 MiB: lists that differ by chance
+// only 0.94 / 0.97 / 1.01 / 1.03 / 1.11 / 1.11 of the time, lists of which some
+// are six times as long 0.70 / 0.73 / 0.66 / 0.80 / 0.75 / 0.82: the line is where
+// the first kind stops gaining.
 constexpr int kSortItems = 4096, kSortBins = 1024, kSortRounds = 32;
 constexpr int64_t kSortKvBytes = 96ll << 20;
 struct FwdSort {
@@ -117,8 +123,15 @@ struct FwdSmem {
   // it is written again.
   int32_t k_rows[kRowSlots];
   int32_t mine[kSortRounds];   // this CTA's items, where they are sorted
-  float m_row[2][kBM];         // row maximum used by tile (tile & 1)
-  float l_row[2][kBM];         // normaliser handed over, per item & 1
+  // row maximum used by tile (tile & 1): tile n + 2 writes it after its warp has read
+  // the maximum of tile n + 1, published after that tile's warp had read tile n's
+  float m_row[2][kBM];
+  // normaliser handed over, per item & 1.  Item i + 2's comes after item i's was
+  // read: since item i the warpgroup that hands over has either finished item i +
+  // 1, and waited there for the other's half, handed over after the epilogue of
+  // item i; or the other finished item i + 1 too, and the first tile of item i + 2,
+  // here, has waited for the maximum of that item's last tile, published after it.
+  float l_row[2][kBM];
   uint32_t tmem_base;
   int abort_flag;
 };
